@@ -4,9 +4,9 @@
 // Design: instead of one radix sort of D 64-bit (tile, depth) keys, the
 // listed Gaussians are first sorted by their 32-bit depth bits (4 onesweep
 // passes over the N_s survivors; the first pass also compacts them out of
-// the N-long footprint arrays), then expanded to one (tile, index) entry per
-// covered tile in depth order, then stably sorted by tile id (1-2 passes
-// over D entries).  Stability gives every tile's list in (depth, index)
+// the N-long footprint arrays); the tile lists then come from that order by
+// one counting sort by tile that never stores the D (tile, index) pairs
+// (bin_tiles.cu).  Stability gives every tile's list in (depth, index)
 // order, exactly the order of a (tile, depth, index) sort.
 //
 // Onesweep pass (single-pass LSD radix step): each CTA takes a 2048-item
@@ -24,19 +24,11 @@
 #include <algorithm>
 #include <string>
 
+#include "bin_tiles.cuh"
 #include "common.cuh"
 #include "sort.cuh"
 
 namespace msgs {
-
-constexpr int kDupThreads = 256;
-constexpr int kDupIPT = 4;
-constexpr int kDupPart = kDupThreads * kDupIPT;
-constexpr int kDupRun = 8;                      // entries one thread emits per window
-constexpr int kDupWin = kDupThreads * kDupRun;  // entries staged per window
-constexpr unsigned long long kDupFlagAgg = 1ull << 62;
-constexpr unsigned long long kDupFlagPre = 2ull << 62;
-constexpr unsigned long long kDupValMask = (1ull << 62) - 1;
 
 __device__ __forceinline__ uint32_t lanemask_lt() {
     uint32_t m;
@@ -83,6 +75,7 @@ __device__ __forceinline__ uint64_t pass_count(const PassArgs &a) {
 template <int IPT>
 __global__ void __launch_bounds__(kSortThreads)
 onesweep_pass(PassArgs a) {
+    pdl_wait();
     constexpr int kPart = SortCfg<IPT>::kPart;
     extern __shared__ __align__(16) uint32_t sort_smem[];
     uint32_t(*s_whist)[kDigits] = reinterpret_cast<uint32_t(*)[kDigits]>(sort_smem);
@@ -235,261 +228,8 @@ onesweep_pass(PassArgs a) {
     }
 }
 
-// Duplication: exclusive scan of n_tiles in depth order (decoupled look-back
-// across partitions), then one (tile id, Gaussian index) entry per covered
-// tile, emitted with a block-wide load-balanced search so writes are
-// contiguous.  Also accumulates the tile-id digit histograms of the
-// following radix passes.
-struct DupArgs {
-    const uint32_t *order;       // Gaussian indices in depth order
-    const uint32_t *n_tiles;
-    const uint2 *rect;
-    const uint32_t *n32;         // survivors (device)
-    uint64_t n_max;              // length of n_tiles / rect
-    int tiles_x;
-    uint32_t tiles;
-    uint64_t cap;
-    uint32_t *keys_out, *vals_out;
-    uint32_t *hist;              // [2][256]
-    unsigned long long *status;  // [partitions]
-    uint32_t *ticket;
-    unsigned long long *err;
-    const unsigned long long *dup;  // duplicates D (device)
-    uint32_t *tstatus;           // tile-pass look-back words, zeroed here
-    uint64_t tstride;            // words per tile pass in tstatus
-    uint32_t tpart;              // partition size of the tile passes
-    uint32_t spin_limit;         // look-back polls before a wait gives up
-};
-
-// kSparse: the order may hold Gaussians without tiles in this frame (a depth
-// order shared by several frames); their rectangles are not loaded.
-template <bool kSparse>
-__global__ void __launch_bounds__(kDupThreads)
-duplicate_kernel(DupArgs a) {
-    __shared__ uint32_t s_off[kDupPart + 1];
-    __shared__ uint32_t s_idx[kDupPart];
-    __shared__ uint2 s_rect[kDupPart];
-    __shared__ uint32_t s_hist[2][256];
-    __shared__ uint2 s_emit[kDupWin];
-    __shared__ uint32_t s_warp[kSortWarps];
-    __shared__ uint32_t s_part;
-    __shared__ unsigned long long s_prefix;
-    const int tid = threadIdx.x;
-    const uint64_t n = umin64(*a.n32, a.n_max);
-    const uint64_t parts = (n + kDupPart - 1) / kDupPart;
-    for (int i = tid; i < 512; i += kDupThreads) (&s_hist[0][0])[i] = 0;
-    {
-        // clear the look-back words the tile passes will use (only as many
-        // partitions as D needs; the passes start after this kernel ends)
-        const uint64_t words = ((umin64(*a.dup, a.cap) + a.tpart - 1) / a.tpart) * 256;
-        for (uint64_t w = blockIdx.x * (uint64_t)kDupThreads + tid; w < words;
-             w += (uint64_t)gridDim.x * kDupThreads) {
-            a.tstatus[w] = 0u;
-            a.tstatus[a.tstride + w] = 0u;
-        }
-    }
-    for (;;) {
-        __syncthreads();
-        if (tid == 0) s_part = atomicAdd(a.ticket, 1u);
-        __syncthreads();
-        const uint32_t p = s_part;
-        if (p >= parts) break;
-        uint32_t nt[kDupIPT], gi[kDupIPT];
-        uint32_t sum = 0;
-#pragma unroll
-        for (int r = 0; r < kDupIPT; r++) {
-            const uint64_t j = (uint64_t)p * kDupPart + tid * kDupIPT + r;
-            gi[r] = j < n ? a.order[j] : 0xffffffffu;
-        }
-#pragma unroll
-        for (int r = 0; r < kDupIPT; r++) {
-            const uint32_t g = gi[r];
-            uint32_t c = 0;
-            uint2 rc = make_uint2(0, 0);
-            if (g != 0xffffffffu) {
-                if (g < a.n_max) {
-                    c = a.n_tiles[g];
-                    if (!kSparse || c) rc = a.rect[g];
-                } else {
-                    MS_DCHECK(false, a.err);
-                    atomicOr(a.err, (unsigned long long)kStatusTimeout);
-                }
-            }
-            s_idx[tid * kDupIPT + r] = g;
-            s_rect[tid * kDupIPT + r] = rc;
-            nt[r] = c;
-            sum += c;
-        }
-        uint32_t total;
-        uint32_t excl = block_excl_scan256(sum, s_warp, total);
-#pragma unroll
-        for (int r = 0; r < kDupIPT; r++) {
-            s_off[tid * kDupIPT + r] = excl;
-            excl += nt[r];
-        }
-        if (tid == 0) {
-            s_off[kDupPart] = total;
-            unsigned long long *st = a.status + p;
-            unsigned long long pre = 0;
-            if (p == 0) {
-                st_relaxed64(st, kDupFlagPre | total);
-            } else {
-                st_relaxed64(st, kDupFlagAgg | total);
-                // batched look-back over up to kLookback predecessors
-                int64_t k = (int64_t)p - 1;
-                uint32_t spins = 0;
-                while (k >= 0) {
-                    unsigned long long v[kLookback];
-#pragma unroll
-                    for (int i = 0; i < kLookback; i++)
-                        v[i] = (k - i >= 0) ? ld_relaxed64(a.status + (k - i)) : kDupFlagPre;
-                    int i = 0;
-                    bool stop = false;
-                    for (; i < kLookback; i++) {
-                        if ((v[i] >> 62) == 0) break;
-                        pre += v[i] & kDupValMask;
-                        if (v[i] & kDupFlagPre) {
-                            stop = true;
-                            break;
-                        }
-                    }
-                    if (stop) break;
-                    k -= i;
-                    if (i == 0) {
-                        if (++spins > a.spin_limit) {
-                            atomicOr(a.err, (unsigned long long)kStatusTimeout);
-                            break;
-                        }
-                        __nanosleep(32);
-                    }
-                }
-                st_relaxed64(st, kDupFlagPre | ((pre + total) & kDupValMask));
-            }
-            s_prefix = pre;
-        }
-        __syncthreads();
-        const uint64_t base = s_prefix;
-        // emission in windows of kDupWin entries: each thread builds a run of
-        // kDupRun consecutive entries (one search for the run's first item,
-        // then it steps through the items' tile rectangles), the window is
-        // staged in shared memory and written out coalesced
-        for (uint32_t w0 = 0; w0 < total; w0 += kDupWin) {
-            const uint32_t k0 = w0 + (uint32_t)tid * kDupRun;
-            if (k0 < total) {
-                // last item whose offset is <= k0
-                int lo = 0, hi = kDupPart;  // invariant s_off[lo] <= k0 < s_off[hi]
-                while (hi - lo > 1) {
-                    int mid = (lo + hi) >> 1;
-                    if (s_off[mid] <= k0) lo = mid;
-                    else hi = mid;
-                }
-                uint2 rc = s_rect[lo];
-                uint32_t x0 = rc.x & 0xffffu, y0 = rc.x >> 16;
-                uint32_t w = (rc.y & 0xffffu) - x0 + 1;
-                const uint32_t m = k0 - s_off[lo];
-                uint32_t xx = m % w, yy = m / w;
-                uint32_t hb = 0xffffffffu, hc = 0;  // run of equal high bytes
-#pragma unroll 4
-                for (int r = 0; r < kDupRun; r++) {
-                    const uint32_t k = k0 + r;
-                    if (k >= total) break;
-                    while (k >= s_off[lo + 1]) {  // next item with tiles
-                        lo++;
-                        rc = s_rect[lo];
-                        x0 = rc.x & 0xffffu;
-                        y0 = rc.x >> 16;
-                        w = (rc.y & 0xffffu) - x0 + 1;
-                        xx = 0;
-                        yy = 0;
-                    }
-                    uint32_t tile = (y0 + yy) * (uint32_t)a.tiles_x + x0 + xx;
-                    if (++xx == w) {
-                        xx = 0;
-                        yy++;
-                    }
-                    if (tile >= a.tiles) {
-                        MS_DCHECK(false, a.err);
-                        atomicOr(a.err, (unsigned long long)kStatusTimeout);
-                        tile = 0xffffffffu;  // not written
-                    } else if (base + k < a.cap) {  // the entries the tile passes sort
-                        atomicAdd(&s_hist[0][tile & 255u], 1u);
-                        const uint32_t h = (tile >> 8) & 255u;
-                        if (h != hb) {
-                            if (hc) atomicAdd(&s_hist[1][hb], hc);
-                            hb = h;
-                            hc = 0;
-                        }
-                        hc++;
-                    }
-                    s_emit[tid * kDupRun + r] = make_uint2(tile, s_idx[lo]);
-                }
-                if (hc) atomicAdd(&s_hist[1][hb], hc);
-            }
-            __syncthreads();
-            const uint32_t cnt = min(total - w0, (uint32_t)kDupWin);
-            for (uint32_t j = tid; j < cnt; j += kDupThreads) {
-                const uint2 e = s_emit[j];
-                const uint64_t g = base + w0 + j;
-                if (e.x == 0xffffffffu) continue;  // reported above
-                if (g < a.cap) {
-                    a.keys_out[g] = e.x;
-                    a.vals_out[g] = e.y;
-                } else {
-                    atomicOr(a.err, (unsigned long long)kStatusOverflow);
-                }
-            }
-            __syncthreads();
-        }
-    }
-    __syncthreads();
-    for (int i = tid; i < 512; i += kDupThreads) {
-        uint32_t v = (&s_hist[0][0])[i];
-        if (v) atomicAdd(&a.hist[i], v);
-    }
-}
-
-// [start, end) of every tile's run in the tile-sorted keys.  Each thread
-// takes 8 consecutive keys (two 16-byte loads when the keys are 16-byte
-// aligned) and the key on either side, all loaded before any is compared,
-// so a thread has several loads in flight instead of one per key.
-constexpr uint32_t kNoTile = 0xffffffffu;
-__global__ void ranges_kernel(const uint32_t *__restrict__ keys,
-                              const unsigned long long *__restrict__ dup, uint64_t cap,
-                              uint32_t tiles, uint32_t *__restrict__ ranges) {
-    const uint64_t n = umin64(*dup, cap);
-    const uint64_t chunks = (n + 7) / 8;
-    const bool vec = (reinterpret_cast<uintptr_t>(keys) & 15u) == 0;
-    for (uint64_t c = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; c < chunks;
-         c += (uint64_t)gridDim.x * blockDim.x) {
-        const uint64_t base = c * 8;
-        uint32_t k[8];
-        if (vec && base + 8 <= n) {
-            const uint4 a = __ldg(reinterpret_cast<const uint4 *>(keys + base));
-            const uint4 b = __ldg(reinterpret_cast<const uint4 *>(keys + base) + 1);
-            k[0] = a.x; k[1] = a.y; k[2] = a.z; k[3] = a.w;
-            k[4] = b.x; k[5] = b.y; k[6] = b.z; k[7] = b.w;
-        } else {
-#pragma unroll
-            for (int j = 0; j < 8; j++) k[j] = base + j < n ? __ldg(keys + base + j) : kNoTile;
-        }
-        const uint32_t prev = base > 0 ? __ldg(keys + base - 1) : kNoTile;
-        const uint32_t next = base + 8 < n ? __ldg(keys + base + 8) : kNoTile;
-#pragma unroll
-        for (int j = 0; j < 8; j++) {
-            const uint32_t kk = k[j];
-            if (kk >= tiles) continue;  // also the positions past n
-            const uint32_t left = j == 0 ? prev : k[j - 1];
-            const uint32_t right = j == 7 ? next : k[j + 1];
-            const uint32_t i = (uint32_t)(base + j);
-            if (left != kk) ranges[2 * (uint64_t)kk] = i;
-            if (right != kk) ranges[2 * (uint64_t)kk + 1] = i + 1;
-        }
-    }
-}
-
-// The first kernel of ms_bin: zeroes the workspace's look-back words,
-// tickets and histograms and the caller's tile ranges (grid-stride, 16-byte
-// stores where aligned), and thread 0 writes the counts: D and the survivors
+// The first kernel of ms_bin: zeroes the workspace's look-back words and
+// tickets (grid-stride, 16-byte stores), and thread 0 writes the counts: D and the survivors
 // from the projection's stats, the status word with the overflow bit, the
 // projection's own status and (ms_bin_ordered) the status of the depth sort
 // it takes its order from.  Every later kernel of the call only ORs into
@@ -497,12 +237,11 @@ __global__ void ranges_kernel(const uint32_t *__restrict__ keys,
 __global__ void bin_start_kernel(const uint32_t *__restrict__ stats,
                                  const uint32_t *__restrict__ order_stats,
                                  unsigned long long *__restrict__ counts, uint64_t cap,
-                                 uint4 *__restrict__ zero16, uint64_t n16,
-                                 uint32_t *__restrict__ ranges, uint64_t n_ranges) {
+                                 uint4 *__restrict__ zero16, uint64_t n16) {
+    pdl_wait();
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     const uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
     for (uint64_t i = t; i < n16; i += stride) zero16[i] = make_uint4(0u, 0u, 0u, 0u);
-    for (uint64_t i = t; i < n_ranges; i += stride) ranges[i] = 0u;
     if (t == 0) {
         const unsigned long long d = *reinterpret_cast<const unsigned long long *>(stats + kStatDup);
         unsigned long long st = stats[kStatStatus];
@@ -526,8 +265,8 @@ static int launch_pass(const PassArgs &a, uint64_t bound, cudaStream_t st) {
     const int per_sm = a.ctas_per_sm > 0 ? a.ctas_per_sm
                        : bound <= kSmallPassItems ? kSmallPassCtasPerSm : kLargePassCtasPerSm;
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(parts, (int64_t)num_sms() * per_sm));
-    onesweep_pass<IPT><<<grid, kSortThreads, SortCfg<IPT>::kSmem, st>>>(a);
-    return MS_OK;
+    return cuda_check(launch_after(onesweep_pass<IPT>, grid, kSortThreads, SortCfg<IPT>::kSmem, st, a),
+                      "onesweep launch");
 }
 
 int launch_onesweep(const PassArgs &a, uint64_t bound, cudaStream_t st) {
@@ -695,21 +434,23 @@ __global__ void __launch_bounds__(kSplitThreads) split_kernel(SplitArgs a) {
 
 struct BinLayout {
     size_t dkeys_a, dvals_a, dkeys_b, dvals_b;
-    size_t tkeys_a, tvals_a, tkeys_b, tvals_b;
+    size_t matrix;      // the tile stage's counts, up to zero_begin
     size_t zero_begin;  // everything from here to total is zeroed per call
-    size_t tickets, thist, dup_status, dstatus, tstatus;
+    size_t tickets, tile_sums, block_sums, dstatus;
     size_t total;
-    int64_t dparts, tparts, dupparts;
+    int64_t dparts;
 };
 
 static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
+// 16 bytes per Gaussian for the depth passes' key / index pairs, then
+// 16 bytes and about one more per tile-list entry for the tile stage's
+// matrix (bin_tiles.cu cuts the entries into as many chunks as it holds
+// rows), then the zeroed words.
 static bool layout(int64_t n, int64_t cap, BinLayout &L) {
     if (n < 0 || n > kMaxSortItems || cap < 1 || cap > kMaxSortItems) return false;
     int64_t nn = n > 0 ? n : 1;
     L.dparts = sort_parts((uint64_t)nn);
-    L.tparts = sort_parts((uint64_t)cap);
-    L.dupparts = ceil_div(nn, kDupPart);
     size_t o = 0;
     auto take = [&](size_t bytes) {
         size_t at = o;
@@ -720,15 +461,12 @@ static bool layout(int64_t n, int64_t cap, BinLayout &L) {
     L.dvals_a = take(nn * 4);
     L.dkeys_b = take(nn * 4);
     L.dvals_b = take(nn * 4);
-    L.tkeys_a = take(cap * 4);
-    L.tvals_a = take(cap * 4);
-    L.tkeys_b = take(cap * 4);
-    L.tvals_b = take(cap * 4);
-    L.tstatus = take((size_t)2 * L.tparts * 256 * 4);  // cleared by duplicate_kernel
+    L.matrix = take(4 * align256(cap * 4));
+    take((size_t)2 * sort_parts((uint64_t)cap) * 256 * 4);
     L.zero_begin = o;
     L.tickets = take(16 * 4);
-    L.thist = take(512 * 4);
-    L.dup_status = take(L.dupparts * 8);
+    L.tile_sums = take(kMaxColBlocks * 4);
+    L.block_sums = take(ceil_div(nn, 1024) * 8);  // >= tile_block_count(nn)
     L.dstatus = take((size_t)4 * L.dparts * 256 * 4);
     L.total = o;
     return true;
@@ -827,17 +565,18 @@ int bin_impl(const ms_proj_t *proj, int64_t n, const ms_camera_t *cam, const ms_
     unsigned long long *err = reinterpret_cast<unsigned long long *>(out->counts) + kCntStatus;
     const uint32_t spin_limit = bin_spin_limit();
 
-    // the zeroed region starts and ends on 256-byte boundaries (layout)
-    const uint64_t n16 = (L.total - L.zero_begin) / 16;
-    bin_start_kernel<<<std::max(1, std::min(sms * 2, (int)ceil_div((int64_t)n16, 256))), 256, 0,
-                       st>>>(proj->stats, order ? order_stats : nullptr,
-                             reinterpret_cast<unsigned long long *>(out->counts),
-                             (uint64_t)out->dup_capacity,
-                             reinterpret_cast<uint4 *>(w + L.zero_begin), n16, out->ranges,
-                             (uint64_t)tiles * 2);
+    // the zeroed region starts and ends on 256-byte boundaries (layout); a
+    // given order needs none of the depth passes' look-back words
+    const uint64_t n16 = ((order ? L.dstatus : L.total) - L.zero_begin) / 16;
+    if ((rc = cuda_check(launch_after(bin_start_kernel,
+                                      std::max(1, std::min(sms * 2, (int)ceil_div((int64_t)n16, 256))),
+                                      256, 0, st, proj->stats, order ? order_stats : nullptr,
+                                      reinterpret_cast<unsigned long long *>(out->counts),
+                                      (uint64_t)out->dup_capacity,
+                                      reinterpret_cast<uint4 *>(w + L.zero_begin), n16),
+                         "bin start")))
+        return rc;
     const uint32_t *survivors = proj->stats + kStatSurvivors;
-    const unsigned long long *dup64 =
-        reinterpret_cast<const unsigned long long *>(proj->stats + kStatDup);
     const uint32_t *order_n = order ? order_stats + kStatSurvivors : survivors;
     if (!order) {
         // ---- depth sort: 4 passes over the listed Gaussians; after them
@@ -845,55 +584,29 @@ int bin_impl(const ms_proj_t *proj, int64_t n, const ms_camera_t *cam, const ms_
         if ((rc = depth_passes(proj, n, L, w, U32(L.dvals_b), err, spin_limit, st))) return rc;
         order = U32(L.dvals_b);
     }
-    // ---- duplicate into (tile, index) entries
-    DupArgs da;
-    da.order = order;
-    da.n_tiles = proj->n_tiles;
-    da.rect = reinterpret_cast<const uint2 *>(proj->rect);
-    da.n32 = order_n;
-    da.n_max = (uint64_t)n;
-    da.tiles_x = tiles_x;
-    da.tiles = (uint32_t)tiles;
-    da.cap = (uint64_t)out->dup_capacity;
-    da.keys_out = U32(L.tkeys_a);
-    da.vals_out = U32(L.tvals_a);
-    da.hist = U32(L.thist);
-    da.status = reinterpret_cast<unsigned long long *>(w + L.dup_status);
-    da.ticket = tickets + 4;
-    da.err = err;
-    da.dup = dup64;
-    da.tstatus = U32(L.tstatus);
-    da.tstride = (uint64_t)L.tparts * 256;
-    da.tpart = (uint32_t)sort_part((uint64_t)out->dup_capacity);
-    da.spin_limit = spin_limit;
-    int dupgrid = (int)std::min<int64_t>(L.dupparts, (int64_t)sms * 4);
-    if (order_stats) duplicate_kernel<true><<<dupgrid, kDupThreads, 0, st>>>(da);
-    else duplicate_kernel<false><<<dupgrid, kDupThreads, 0, st>>>(da);
-    // ---- stable sort by tile id
-    const int tpasses = tiles <= 256 ? 1 : 2;
-    uint32_t *final_keys = U32(L.tkeys_b);
-    for (int pass = 0; pass < tpasses; pass++) {
-        PassArgs a;
-        a.keys_in = pass == 0 ? U32(L.tkeys_a) : U32(L.tkeys_b);
-        a.vals_in = pass == 0 ? U32(L.tvals_a) : U32(L.tvals_b);
-        a.filter = nullptr;
-        bool last = pass == tpasses - 1;
-        a.keys_out = pass == 0 ? U32(L.tkeys_b) : U32(L.tkeys_a);
-        a.vals_out = last ? out->gauss_idx : U32(L.tvals_b);
-        final_keys = a.keys_out;
-        a.n32 = nullptr;
-        a.n64 = dup64;
-        a.n_cap = (uint64_t)out->dup_capacity;
-        a.shift = 8 * pass;
-        a.hist = U32(L.thist) + 256 * pass;
-        a.status = U32(L.tstatus) + (size_t)pass * L.tparts * 256;
-        a.ticket = tickets + 5 + pass;
-        a.err = err;
-        a.spin_limit = spin_limit;
-        if ((rc = launch_onesweep(a, (uint64_t)out->dup_capacity, st))) return rc;
-    }
-    ranges_kernel<<<sms * 4, 256, 0, st>>>(final_keys, dup64, (uint64_t)out->dup_capacity,
-                                           (uint32_t)tiles, out->ranges);
+    // ---- tile lists from the order; the depth passes' buffers but for the
+    // order's own are free now
+    TileListArgs ta;
+    ta.order = order;
+    ta.n32 = order_n;
+    ta.n_tiles = proj->n_tiles;
+    ta.rect = reinterpret_cast<const uint2 *>(proj->rect);
+    ta.n = n;
+    ta.tiles_x = tiles_x;
+    ta.tiles = tiles;
+    ta.cap = out->dup_capacity;
+    ta.gauss_idx = out->gauss_idx;
+    ta.ranges = out->ranges;
+    ta.err = err;
+    ta.block_sums = reinterpret_cast<unsigned long long *>(w + L.block_sums);
+    ta.block_words = U32(L.dkeys_a);
+    ta.item = reinterpret_cast<uint2 *>(w + L.dvals_a);  // dvals_a and dkeys_b
+    ta.idx = U32(L.dvals_b);
+    ta.matrix = U32(L.matrix);
+    ta.matrix_bytes = L.zero_begin - L.matrix;
+    ta.meta = tickets + 8;
+    ta.tile_sums = U32(L.tile_sums);
+    if ((rc = launch_tile_lists(ta, st))) return rc;
     return cuda_check(cudaGetLastError(), "ms_bin launches");
 }
 

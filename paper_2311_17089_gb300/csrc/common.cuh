@@ -110,6 +110,34 @@ __device__ __forceinline__ void fence_acquire() {
     asm volatile("fence.acq_rel.gpu;" ::: "memory");
 }
 
+// Programmatic dependent launch: a kernel launched with launch_after starts
+// while the kernel before it in the stream is still draining, and waits in
+// pdl_wait (the first thing it does, in every thread, so that its own end
+// implies its predecessors') until that kernel has ended and its writes are
+// visible.  pdl_wait also lets the next kernel's launch begin.  Between the
+// dozen short dependent kernels of a frame this hides the launch and the
+// CTAs' start, 1-3 us each.
+__device__ __forceinline__ void pdl_wait() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+template <typename... P, typename... A>
+inline cudaError_t launch_after(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
+                                cudaStream_t st, A &&...args) {
+    cudaLaunchConfig_t c = {};
+    c.gridDim = grid;
+    c.blockDim = block;
+    c.dynamicSmemBytes = smem;
+    c.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = at;
+    c.numAttrs = 1;
+    return cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
+}
+
 inline int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }
 int num_sms();
 // cudaFuncAttributeMaxDynamicSharedMemorySize = bytes for func on the
