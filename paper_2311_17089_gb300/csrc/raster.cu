@@ -8,8 +8,20 @@
 // resident CTAs) entries; only tiles longer than a fair share of the work
 // are split.
 // A CTA walks its segment in sub-batches of kChunk records, double-buffered:
-// the next sub-batch arrives in shared memory by per-record bulk copies
-// (cp.async.bulk) on an mbarrier while the current one is blended.
+// the next sub-batch arrives in shared memory (cp.async, a record per
+// thread, on an mbarrier) while the current one is blended.  A sub-batch's
+// records are first tested against the tile's sixteen 4x4 pixel blocks; each
+// half warp then blends only those that reach its block, four at a time.
+//
+// Bound by instruction issue where the SMs are full (1256x832: 175M warp
+// instructions, 74% of the issue slots), by a deep tile's serial walk where
+// they are not.  GB300, kernel times before (8x4 blocks by box test, record
+// pairs regrouped through shared memory, per-record bulk copies) and now:
+// 1256x832 of 1M Gaussians 242 -> 206 us, 628x416 at all levels 88 -> 72,
+// 256x256 of 10k 42 -> 38, near/far 3M 700 -> 631.  The copies alone made
+// 241 -> 219 and 820 -> 726 (the bulk engine takes 48-byte copies one by
+// one).  Two pixels per thread (8x8 blocks per warp, packed arithmetic)
+// issued as much and lengthened the deep walks (3M: 870 to 1130 us).
 //
 // The blend stays exactly sequential across segments (decoupled look-back):
 //   - a segment whose predecessor has published its inclusive prefix
@@ -43,7 +55,6 @@ namespace msgs {
 
 constexpr int kRecBytes = 48;                // one raster record
 constexpr int kBufBytes = kChunk * kRecBytes;  // staged records, as copied
-constexpr int kPairs = kChunk / 2;
 constexpr float kAlphaMax = 0.99f;
 constexpr float kTStop = 1e-4f;
 #ifndef MS_RASTER_WINDOW
@@ -68,6 +79,30 @@ __device__ __forceinline__ float ex2_approx(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
+}
+
+__device__ __forceinline__ float sqrt_approx(float x) {
+    float y;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+// Loads from shared memory at a 32-bit address plus a constant.
+template <int kOff>
+__device__ __forceinline__ float4 lds4(uint32_t p) {
+    float4 v;
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4 + %5];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+                 : "r"(p), "n"(kOff));
+    return v;
+}
+template <int kOff>
+__device__ __forceinline__ float2 lds2(uint32_t p) {
+    float2 v;
+    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2 + %3];"
+                 : "=f"(v.x), "=f"(v.y)
+                 : "r"(p), "n"(kOff));
+    return v;
 }
 
 struct RasterArgs {
@@ -98,12 +133,17 @@ struct Seg {
     uint32_t t, k, nk, start, len;
 };
 
+// Segment c's tile and list entries; called by whole warps, whose lanes
+// search together.
 __device__ __forceinline__ Seg seg_of(const RasterArgs &a, uint32_t c, uint32_t L) {
-    int lo = 0, hi = a.tiles;  // seg_off[lo] <= c < seg_off[hi]
-    while (hi - lo > 1) {
-        int mid = (lo + hi) >> 1;
-        if (a.seg_off[mid] <= c) lo = mid;
-        else hi = mid;
+    const uint32_t lane = threadIdx.x & 31u;
+    uint32_t lo = 0, hi = (uint32_t)a.tiles;  // seg_off[lo] <= c < seg_off[hi]
+    while (hi - lo > 1u) {
+        const uint32_t step = (hi - lo + 31u) / 32u, q = lo + (lane + 1u) * step;
+        const uint32_t n =
+            __popc(__ballot_sync(0xffffffffu, q < hi && __ldg(a.seg_off + q) <= c));
+        lo += n * step;
+        hi = min(hi, lo + step);
     }
     Seg sg;
     sg.t = lo;
@@ -189,156 +229,227 @@ struct PixelState {
     bool term;
 };
 
-// One warp's share of a staged sub-batch: the records whose alpha >= 1/255
-// level set can reach the warp's 8x4 pixel block, in list order, regrouped
-// into pairs (2m, 2m+1) with each field of the two records side by side,
-// so one packed FP32x2 instruction evaluates both records' power terms.
-struct WarpPairs {
-    float4 q0[kPairs];     // ux0 ux1 uy0 uy1
-    float4 q1[kPairs];     // A0 A1 B0 B1
-    float4 q2[kPairs];     // C0 C1 thr0 thr1
-    float4 q3[kPairs];     // opacity0 opacity1 r0 r1
-    float4 q4[kPairs];     // g0 g1 b0 b1
-    uint16_t idx[kChunk];  // index of each record within the sub-batch
-};
+// A warp covers an 8x4 block of pixels, each half warp a 4x4 one with its
+// own list of the records that reach it.  (Of the lane slots of an 8x4
+// block's records, about 37% are accepted by their pixel on the 1M-Gaussian
+// scene at 1256x832, of a 4x4 block's half.)
 constexpr int kWarps = kRasterThreads / 32;
-constexpr int kSmemBytes = 2 * kBufBytes + kWarps * (int)sizeof(WarpPairs);
-// Half extents of a warp's block of pixel centres (8 x 4 pixels) plus a
-// margin for FP32 rounding: the record's half extents bound the exact
-// alpha >= 1/255 level set, and the rounding of that bound and of the
-// distances is below 1e-4 px at the largest image coordinates.
+constexpr int kGroup = 4;  // records blended at a time; a list is padded to it
+constexpr int kListLen = kChunk + kGroup;
+// Dynamic shared memory: two staging buffers, a record that no pixel accepts
+// (the lists' padding), the records' block masks, and the half warps' lists.
+constexpr int kMaskOff = 2 * kBufBytes + kRecBytes;
+constexpr int kListOff = kMaskOff + kChunk * 2;
+constexpr int kSmemBytes = kListOff + kWarps * 2 * kListLen * 2;
+// A record's half extents bound the exact alpha >= 1/255 level set; the
+// rounding of that bound, of the chords below and of the distances is below
+// 1e-3 px at the largest image coordinates.
 #ifndef MS_CULL_MARGIN
 #define MS_CULL_MARGIN 0.0625f
 #endif
-constexpr float kBlockHalfX = 3.5f + MS_CULL_MARGIN;
-constexpr float kBlockHalfY = 1.5f + MS_CULL_MARGIN;
+constexpr float kInf = __builtin_huge_valf();
 
-// Compact the records [0, cnt) of the staged sub-batch whose level-set box
-// (centre +- (ex, ey)) can reach the warp's block of pixel centres
-// (centre (cx, cy)) into the warp's pair buffer, keeping list order.  Any
-// other record has alpha < 1/255 at every pixel of the block, so skipping
-// it changes nothing.  An odd count is padded with a record that no pixel
-// accepts (thr = +inf).  Returns the count (warp-uniform).
-__device__ __forceinline__ uint32_t compact(const float4 *__restrict__ aos, uint32_t cnt,
-                                            float cx, float cy, WarpPairs &wp) {
-    const uint32_t lane = threadIdx.x & 31u;
-    uint32_t base = 0;
+// Bits 4 k + j, k = 0, 1: some pixel centre of the tile's 4x4 block (j, row
+// band b0 + k) may have alpha >= 1/255.  (x, y): the record's centre relative
+// to the tile's corner.  Over a band of pixel rows the level set {A dx^2 +
+// B dx dy + C dy^2 >= thr} spans an x interval whose ends are chords' ends:
+// the right end is largest at the row of the set's rightmost point (dx = ex,
+// dy = -B ex / 2C), so over the band at the nearest row to that; the left
+// end likewise with the signs turned.  The discriminant is raised by more
+// than its rounding; a conic without usable curvature, or NaN, keeps every
+// block that the box reaches.
+__device__ __forceinline__ uint32_t blocks_reached(float x, float y, float A, float B, float C,
+                                                   float thr, float ex, float ey, int b0) {
+    const float yr = -0.5f * ex * __fdividef(B, C);  // dy of the rightmost point
+    const float ia = __fdividef(-0.5f, A);
+    const bool flat = !(A < -1e-30f) || !(C < -1e-30f);
+    uint32_t bits = 0u;
+#pragma unroll
+    for (int k = 0; k < 2; k++) {
+        // the band's pixel centres relative to the record's
+        const float yl = (float)(4 * (b0 + k)) + 0.5f - y, yh = yl + 3.0f;
+        if (yl > ey + MS_CULL_MARGIN || yh < -ey - MS_CULL_MARGIN) continue;
+        float x1 = ex, x0 = -ex;
+        if (!flat) {
+            auto chord = [&](float dy, float sign) {  // the end of the chord at dy
+                const float h = B * dy, t = 4.0f * A * (C * dy * dy - thr);
+                const float d = h * h - t + 3.8e-6f * (h * h + fabsf(4.0f * A * C * dy * dy) + fabsf(4.0f * A * thr));
+                return ia * (h + sign * sqrt_approx(fmaxf(d, 0.0f)));
+            };
+            const float r = fminf(yh, fmaxf(yl, yr)), l = fminf(yh, fmaxf(yl, -yr));
+            if (r != yr) x1 = chord(r, 1.0f);
+            if (l != -yr) x0 = chord(l, -1.0f);
+        }
+        x1 += x + MS_CULL_MARGIN;
+        x0 += x - MS_CULL_MARGIN;
+#pragma unroll
+        for (int j = 0; j < 4; j++)
+            if (!(4.0f * j + 0.5f > x1) && !(4.0f * j + 3.5f < x0)) bits |= 1u << (4 * k + j);
+    }
+    return bits;
+}
+
+// The records of the staged sub-batch whose block mask has the half warp's
+// bit, as byte offsets in list order, for both halves of the warp (bits
+// `bit` and bit + 1), padded with the record at `pad` to a common multiple
+// of kGroup, which is returned.  Any other record has alpha < 1/255 at every pixel of the
+// block, so skipping it changes nothing.
+__device__ __forceinline__ uint32_t compact(const uint16_t *__restrict__ masks, uint32_t bit,
+                                            uint16_t *lists, uint32_t pad) {
+    const uint32_t lane = threadIdx.x & 31u, lt = (1u << lane) - 1u;
+    uint32_t n[2] = {0u, 0u};
 #pragma unroll
     for (int k = 0; k < kChunk / 32; k++) {
         const uint32_t i = (uint32_t)k * 32u + lane;
-        bool rel = false;
-        float4 r0, r2;
-        if (i < cnt) {
-            r0 = aos[3 * i];
-            r2 = aos[3 * i + 2];
-            rel = fabsf(r0.x - cx) <= r2.z + kBlockHalfX && fabsf(r0.y - cy) <= r2.w + kBlockHalfY;
+        const uint32_t bits = (uint32_t)masks[i] >> bit;
+#pragma unroll
+        for (int h = 0; h < 2; h++) {
+            const uint32_t m = __ballot_sync(0xffffffffu, (bits >> h) & 1u);
+            if ((bits >> h) & 1u) lists[h * kListLen + n[h] + __popc(m & lt)] = (uint16_t)(i * kRecBytes);
+            n[h] += __popc(m);
         }
-        const uint32_t m = __ballot_sync(0xffffffffu, rel);
-        if (rel) {
-            const float4 r1 = aos[3 * i + 1];
-            const uint32_t p = base + __popc(m & ((1u << lane) - 1u));
-            const uint32_t q = p >> 1, h = p & 1u;
-            float *q0 = reinterpret_cast<float *>(&wp.q0[q]);
-            float *q1 = reinterpret_cast<float *>(&wp.q1[q]);
-            float *q2 = reinterpret_cast<float *>(&wp.q2[q]);
-            float *q3 = reinterpret_cast<float *>(&wp.q3[q]);
-            float *q4 = reinterpret_cast<float *>(&wp.q4[q]);
-            q0[h] = r0.x;
-            q0[2 + h] = r0.y;
-            q1[h] = r0.z;
-            q1[2 + h] = r0.w;
-            q2[h] = r1.x;
-            q2[2 + h] = r2.y;
-            q3[h] = r1.y;
-            q3[2 + h] = r1.z;
-            q4[h] = r1.w;
-            q4[2 + h] = r2.x;
-            wp.idx[p] = (uint16_t)i;
-        }
-        base += __popc(m);
     }
-    if ((base & 1u) && lane == 0) {
-        const uint32_t q = base >> 1;
-        float *q0 = reinterpret_cast<float *>(&wp.q0[q]);
-        float *q1 = reinterpret_cast<float *>(&wp.q1[q]);
-        float *q2 = reinterpret_cast<float *>(&wp.q2[q]);
-        float *q3 = reinterpret_cast<float *>(&wp.q3[q]);
-        float *q4 = reinterpret_cast<float *>(&wp.q4[q]);
-        q0[1] = q0[3] = q1[1] = q1[3] = q2[1] = 0.0f;
-        q2[3] = __int_as_float(0x7f800000);
-        q3[1] = q3[3] = q4[1] = q4[3] = 0.0f;
-        wp.idx[base] = 0;
-    }
+    const uint32_t len = (max(n[0], n[1]) + kGroup - 1u) & ~(uint32_t)(kGroup - 1);
+#pragma unroll
+    for (int h = 0; h < 2; h++)
+        for (uint32_t k = n[h] + lane; k < len; k += 32u) lists[h * kListLen + k] = (uint16_t)pad;
     __syncwarp();
-    return base;
+    return len;
 }
 
-// One record's contribution once it passed the alpha test: stop before a
-// Gaussian that would bring T below 1e-4, else accumulate and advance T.
-// Returns true when the pixel terminated.
-__device__ __forceinline__ bool blend_one(float p, float opacity, float r, float g, float b,
-                                          uint32_t pos, PixelState &s) {
-    const float al = fminf(kAlphaMax, opacity * ex2_approx(p));
-    const float Tn = fmaf(-al, s.T, s.T);
+// A pixel being blended: y is its row's centre, or +inf once it has ended
+// (or lies outside the image): every power is then -inf or NaN and no record
+// is accepted.
+struct Pix {
+    float T, C0, C1, C2, y;
+    uint32_t last, evals;
+};
+
+// power * log2(e) = A dx^2 + B dx dy + C dy^2 of a record at the pixel.
+__device__ __forceinline__ float power_of(const float4 r0, float C, float fx, float y) {
+    const float dx = __fsub_rn(fx, r0.x), dy = __fsub_rn(y, r0.y);
+    const float u = __fmaf_rn(r0.w, dy, __fmul_rn(r0.z, dx));
+    return __fmaf_rn(__fmul_rn(C, dy), dy, __fmul_rn(dx, u));
+}
+
+// One record: skipped if the power is positive or alpha below 1/255 (power *
+// log2(e) < thr); stop before a Gaussian that would bring T below 1e-4, else
+// accumulate and advance T.  pos: 1 + its list position.
+__device__ __forceinline__ void blend_one(const float4 *__restrict__ r, float fx, uint32_t pos,
+                                          Pix &s) {
+    const float4 r1 = r[1], r2 = r[2];
+    const float p = power_of(r[0], r1.x, fx, s.y);
+    if (!(p <= 0.0f && p >= r2.y)) return;
+    const float al = fminf(kAlphaMax, __fmul_rn(r1.y, ex2_approx(p)));
+    const float Tn = __fmaf_rn(-al, s.T, s.T);
     if (Tn < kTStop) {
-        s.term = true;
+        s.y = kInf;
         s.evals = pos;
-        return true;
+        return;
     }
-    const float w = al * s.T;
-    s.C0 = fmaf(w, r, s.C0);
-    s.C1 = fmaf(w, g, s.C1);
-    s.C2 = fmaf(w, b, s.C2);
+    const float w = __fmul_rn(al, s.T);
+    s.C0 = __fmaf_rn(w, r1.z, s.C0);
+    s.C1 = __fmaf_rn(w, r1.w, s.C1);
+    s.C2 = __fmaf_rn(w, r2.x, s.C2);
     s.T = Tn;
     s.last = pos;
-    return false;
 }
 
-// Blend the warp's n compacted records of a sub-batch of cnt into s.  pos0
-// is the list position of the sub-batch's first record.  power * log2(e)
-// = A dx^2 + B dx dy + C dy^2 is evaluated for both records of a pair at
-// once; a record is skipped when the power is positive or alpha would stay
-// below 1/255 (power * log2(e) < thr).
-__device__ __forceinline__ void blend_pairs(const WarpPairs &wp, uint32_t n, uint32_t cnt,
-                                            uint32_t pos0, f32x2 fx2, f32x2 fy2, PixelState &s) {
-    const uint32_t np = (n + 1) >> 1;
-#pragma unroll 2
-    for (uint32_t m = 0; m < np; m++) {
-        const ulonglong2 v0 = *reinterpret_cast<const ulonglong2 *>(&wp.q0[m]);
-        const ulonglong2 v1 = *reinterpret_cast<const ulonglong2 *>(&wp.q1[m]);
-        const ulonglong2 v2 = *reinterpret_cast<const ulonglong2 *>(&wp.q2[m]);
-        const f32x2 dx = sub2(fx2, v0.x), dy = sub2(fy2, v0.y);
-        const f32x2 u = fma2(v1.y, dy, mul2(v1.x, dx));
-        const f32x2 pw = fma2(mul2(v2.x, dy), dy, mul2(dx, u));
-        float p0, p1, t0, t1;
-        unpack2(pw, p0, p1);
-        unpack2(v2.y, t0, t1);
-        const bool h0 = p0 <= 0.0f && p0 >= t0;
-        const bool h1 = p1 <= 0.0f && p1 >= t1;
-        if (!(h0 || h1)) continue;
-        const float4 w3 = wp.q3[m], w4 = wp.q4[m];
-        const uint32_t ix = *reinterpret_cast<const uint32_t *>(&wp.idx[2 * m]);
-        if (h0 && blend_one(p0, w3.x, w3.z, w4.x, w4.z, pos0 + (ix & 0xffffu) + 1, s)) return;
-        if (h1 && blend_one(p1, w3.y, w3.w, w4.y, w4.w, pos0 + (ix >> 16) + 1, s)) return;
+// Blend the half warp's listed records (n, the same for both halves) into
+// the thread's pixel; pos0 is the list position of the sub-batch's first
+// record.  kGroup records at a time: all their alphas (0 where not accepted,
+// which leaves T and the colour as they are; independent of T, so their
+// loads and arithmetic overlap), then T through the group and one test
+// whether it ends a pixel of the warp, whose weights are then formed again
+// up to the record that ends it; then the colours.  About 27 instructions a
+// record.  `odd`: some record's colour is not finite (it must not meet a
+// zero weight) or its power may round above 0: one record at a time.
+__device__ __forceinline__ void blend_list(const unsigned char *__restrict__ aos,
+                                           const uint16_t *__restrict__ list, uint32_t n, bool odd,
+                                           uint32_t pos0, float fx, Pix &s) {
+    if (odd) {
+        for (uint32_t m = 0; m < n; m++) {
+            const uint32_t o = list[m];
+            blend_one(reinterpret_cast<const float4 *>(aos + o), fx,
+                      pos0 + o / (uint32_t)kRecBytes + 1u, s);
+        }
+        return;
     }
-    s.evals = pos0 + cnt;
+    const uint32_t base = smem_addr(aos);
+    uint32_t last = 0xffffu;  // offset of the last blended record
+    for (uint32_t m = 0; m < n; m += kGroup) {
+        static_assert(kGroup == 4, "a group's offsets are one 8-byte load");
+        const uint2 ii = *reinterpret_cast<const uint2 *>(list + m);
+        const uint32_t o[kGroup] = {ii.x & 0xffffu, ii.x >> 16, ii.y & 0xffffu, ii.y >> 16};
+        float al[kGroup], w[kGroup], c[kGroup][3];
+#pragma unroll
+        for (int k = 0; k < kGroup; k++) {
+            const uint32_t r = base + o[k];
+            const float4 r1 = lds4<16>(r);
+            const float2 r2 = lds2<32>(r);
+            const float p = power_of(lds4<0>(r), r1.x, fx, s.y);
+            const float a = fminf(kAlphaMax, __fmul_rn(r1.y, ex2_approx(p)));
+            al[k] = p >= r2.y ? a : 0.0f;
+            c[k][0] = r1.z;
+            c[k][1] = r1.w;
+            c[k][2] = r2.x;
+        }
+        float T = s.T;
+#pragma unroll
+        for (int k = 0; k < kGroup; k++) {
+            w[k] = __fmul_rn(al[k], T);
+            T = __fmaf_rn(-al[k], T, T);
+        }
+        const bool ends = T < kTStop;
+        const uint32_t any = __ballot_sync(0xffffffffu, ends);
+        if (any) {
+            if (ends) {
+                T = s.T;
+#pragma unroll
+                for (int k = 0; k < kGroup; k++) {
+                    const float Tn = __fmaf_rn(-al[k], T, T);
+                    if (s.y != kInf && Tn < kTStop) {
+                        s.y = kInf;
+                        s.evals = pos0 + o[k] / (uint32_t)kRecBytes + 1u;
+                    }
+                    const bool on = s.y != kInf;
+                    w[k] = on ? __fmul_rn(al[k], T) : 0.0f;
+                    T = on ? Tn : T;
+                }
+            }
+            __syncwarp();
+        }
+#pragma unroll
+        for (int k = 0; k < kGroup; k++) {
+            s.C0 = __fmaf_rn(w[k], c[k][0], s.C0);
+            s.C1 = __fmaf_rn(w[k], c[k][1], s.C1);
+            s.C2 = __fmaf_rn(w[k], c[k][2], s.C2);
+            if (w[k] != 0.0f) last = o[k];
+        }
+        s.T = T;
+        if (any && !__any_sync(0xffffffffu, s.y != kInf)) break;
+    }
+    if (last != 0xffffu) s.last = pos0 + last / (uint32_t)kRecBytes + 1u;
 }
 
-// Thread 0 arms the buffer's mbarrier with the sub-batch's byte count and
-// every thread issues the bulk copies of its gathered records.  The phase
-// cannot complete before the arming arrival, so no barrier is needed
-// between the two; the caller guarantees that every warp is done reading
-// the buffer.
-__device__ __forceinline__ void issue_batch(const RasterArgs &a, uint32_t first, uint32_t cnt,
+// The first kChunk threads copy their records (g: a thread's list entry)
+// into the buffer and arrive on its mbarrier once their copies have landed
+// (a thread without a record at once); the caller guarantees that every warp
+// is done reading the buffer.
+__device__ __forceinline__ void issue_batch(const RasterArgs &a, uint32_t g, uint32_t cnt,
                                             float4 *buf, uint64_t *bar) {
     MS_DCHECK(cnt <= (uint32_t)kChunk, a.err);
-    if (threadIdx.x == 0) mbar_expect_tx(bar, cnt * kRecBytes);
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    for (uint32_t i = threadIdx.x; i < cnt; i += kRasterThreads) {
-        uint32_t g = a.gidx[first + i];
-        MS_DCHECK(g < a.n_rec, a.err);
-        if (g >= a.n_rec) g = 0;  // unreachable unless binning reported an error
-        bulk_copy_g2s(buf + 3 * i, a.rec + 3 * (size_t)g, kRecBytes, bar);
+    if (threadIdx.x < (uint32_t)kChunk) {
+        if (threadIdx.x < cnt) {
+            MS_DCHECK(g < a.n_rec, a.err);
+            if (g >= a.n_rec) g = 0;  // unreachable unless binning reported an error
+            const float4 *src = a.rec + 3 * (size_t)g;
+            float4 *dst = buf + 3 * threadIdx.x;
+            cp_async16(dst, src);
+            cp_async16(dst + 1, src + 1);
+            cp_async16(dst + 2, src + 2);
+        }
+        cp_async_arrive(bar);
     }
 }
 
@@ -351,18 +462,19 @@ __device__ __forceinline__ bool wait_batch(const RasterArgs &a, uint64_t *bar, u
     return false;
 }
 
-__device__ __forceinline__ PixelState load_state(const float4 *v, const uint2 *v2, uint32_t c) {
-    float4 st = __ldcg(v + (size_t)c * kRasterThreads + threadIdx.x);
-    uint2 st2 = __ldcg(v2 + (size_t)c * kRasterThreads + threadIdx.x);
+// The state of tile pixel slot `i` (fwd_index) after segment c.
+__device__ __forceinline__ PixelState load_state(const float4 *v, const uint2 *v2, uint32_t c,
+                                                 int i) {
+    float4 st = __ldcg(v + (size_t)c * kRasterThreads + i);
+    uint2 st2 = __ldcg(v2 + (size_t)c * kRasterThreads + i);
     PixelState s = {st.x, st.y, st.z, st.w, st2.x, st2.y & ~kTermBit, (st2.y & kTermBit) != 0};
     return s;
 }
 
-__device__ __forceinline__ void store_state(float4 *v, uint2 *v2, uint32_t c,
+__device__ __forceinline__ void store_state(float4 *v, uint2 *v2, uint32_t c, int i,
                                             const PixelState &s) {
-    v[(size_t)c * kRasterThreads + threadIdx.x] = make_float4(s.C0, s.C1, s.C2, s.T);
-    v2[(size_t)c * kRasterThreads + threadIdx.x] =
-        make_uint2(s.last, s.evals | (s.term ? kTermBit : 0u));
+    v[(size_t)c * kRasterThreads + i] = make_float4(s.C0, s.C1, s.C2, s.T);
+    v2[(size_t)c * kRasterThreads + i] = make_uint2(s.last, s.evals | (s.term ? kTermBit : 0u));
 }
 
 // The exact state after one more segment, from the state P before it and
@@ -392,25 +504,34 @@ __device__ __forceinline__ uint32_t ld_volatile(const uint32_t *p) {
 }
 
 // Walk one segment in sub-batches through two staging buffers: while the
-// warps compact and blend sub-batch j from one buffer, the bulk copies of
-// sub-batch j + 1 land in the other.  One CTA barrier per sub-batch (the
-// termination count) also guarantees that every warp has compacted
-// sub-batch j before sub-batch j + 2 is copied over it.  In local mode
-// (`exact` false) the walk stops as soon as the tile is marked done.  The
-// CTA stops early once every pixel has terminated.  Returns kWalked,
-// kAborted.  A copy wait that gives up sets the status word and ends the
-// waiting warps' pixels; the walk stays in step across the CTA.
+// warps mask, list and blend the records of sub-batch j in one buffer, the
+// bulk copies of sub-batch j + 1 land in the other and the list entries of
+// sub-batch j + 2 are read.  Two CTA barriers per sub-batch: after the block
+// masks, and with the termination test, when every warp is done with
+// sub-batch j.  In local mode (`exact` false) the walk stops as soon as the
+// tile is marked done.  The CTA stops early once every pixel has
+// terminated.  Returns kWalked, kAborted.  A copy wait that gives up sets
+// the status word and ends the waiting warps' pixels; the walk stays in
+// step across the CTA.
 constexpr int kWalked = 0, kAborted = 1;
 __device__ __forceinline__ int run_segment(const RasterArgs &a, const Seg &sg, uint32_t L,
-                                            bool exact, bool inside, float fx, float fy,
-                                            float cx, float cy, PixelState &s,
-                                            float4 *aos, WarpPairs &wp, uint64_t *bar,
-                                            uint32_t &par, uint32_t *s_abort) {
+                                           bool exact, bool active, float fx, float fy, int tx,
+                                           int ty, PixelState &s, unsigned char *smem,
+                                           uint64_t *bar, uint32_t &par, uint32_t *s_abort) {
     const uint32_t pos0 = sg.k * L;
     if (sg.len == 0) return kWalked;
     const uint32_t nb = (sg.len + kChunk - 1) / kChunk;
-    const f32x2 fx2 = pack2(fx, fx), fy2 = pack2(fy, fy);
-    issue_batch(a, sg.start, min(sg.len, (uint32_t)kChunk), aos, &bar[0]);
+    const uint32_t tid = threadIdx.x, wid = tid >> 5;
+    float4 *aos = reinterpret_cast<float4 *>(smem);
+    unsigned char *masks = smem + kMaskOff;
+    uint16_t *lists = reinterpret_cast<uint16_t *>(smem + kListOff) + wid * 2u * kListLen;
+    auto entry = [&](uint32_t j) {  // this thread's list entry of sub-batch j
+        const uint32_t i = j * kChunk + tid;
+        return tid < (uint32_t)kChunk && i < sg.len ? __ldg(a.gidx + sg.start + i) : 0u;
+    };
+    Pix q = {s.T, s.C0, s.C1, s.C2, active && !s.term ? fy : kInf, s.last, s.evals};
+    issue_batch(a, entry(0), min(sg.len, (uint32_t)kChunk), aos, &bar[0]);
+    uint32_t next = entry(1);
     bool abort = false;
     for (uint32_t j = 0; j < nb; j++) {
         const uint32_t b = j & 1u, off = j * kChunk;
@@ -418,24 +539,48 @@ __device__ __forceinline__ int run_segment(const RasterArgs &a, const Seg &sg, u
         const bool ok = wait_batch(a, &bar[b], (par >> b) & 1u);
         par ^= 1u << b;
         const bool more = j + 1 < nb;
-        if (more)
-            issue_batch(a, sg.start + off + kChunk, min(sg.len - off - kChunk, (uint32_t)kChunk),
+        if (more) {
+            issue_batch(a, next, min(sg.len - off - kChunk, (uint32_t)kChunk),
                         aos + (b ^ 1u) * 3 * kChunk, &bar[b ^ 1u]);
+            next = entry(j + 2);
+        }
         // a copy wait that gave up has set the status word: the warp's pixels
         // stop here (their result is reported wrong), the walk goes on in
         // step with the other warps
-        const bool wok = __all_sync(0xffffffffu, ok);
-        if (!wok) s.term = true;
+        if (!__all_sync(0xffffffffu, ok)) q.y = kInf;
+        // the block masks: a thread takes one record and two of the tile's
+        // four row bands
+        const float4 *buf = aos + b * 3 * kChunk;
+        bool bad = false;
+        {
+            const uint32_t i = tid & (uint32_t)(kChunk - 1), band = (tid / kChunk) * 2u;
+            uint32_t bits = 0u;
+            if (i < cnt) {
+                const float4 r0 = buf[3 * i], r1 = buf[3 * i + 1], r2 = buf[3 * i + 2];
+                bits = blocks_reached(r0.x - (float)(tx * 16), r0.y - (float)(ty * 16), r0.z, r0.w,
+                                      r1.x, r2.y, r2.z, r2.w, (int)band);
+                // B^2 below 4 A C by more than the power's rounding, a few
+                // 2^-24 of its terms: it cannot come out positive
+                bad = !((r1.z + r1.w + r2.x) * 0.0f == 0.0f) ||
+                      !(r0.w * r0.w < 3.99998474f * r0.z * r1.x);
+            }
+            masks[2u * i + tid / kChunk] = (unsigned char)bits;
+        }
+        const bool odd = __syncthreads_or(bad) != 0;
         // warps whose pixels have all terminated skip their share
-        const bool wlive = wok && __any_sync(0xffffffffu, inside && !s.term);
-        const uint32_t nw = wlive ? compact(aos + b * 3 * kChunk, cnt, cx, cy, wp) : 0u;
-        if (wlive && inside && !s.term) blend_pairs(wp, nw, cnt, pos0 + off, fx2, fy2, s);
+        if (__any_sync(0xffffffffu, q.y != kInf)) {
+            const uint32_t n = compact(reinterpret_cast<const uint16_t *>(masks),
+                                       (wid >> 1) * 4u + (wid & 1u) * 2u, lists, (2u - b) * kBufBytes);
+            blend_list(reinterpret_cast<const unsigned char *>(buf),
+                       lists + ((tid >> 4) & 1u) * kListLen, n, odd, pos0 + off, fx, q);
+            if (q.y != kInf) q.evals = pos0 + off + cnt;
+        }
         // two slots: a warp may still be reading sub-batch j's value while
-        // thread 0 writes sub-batch j + 1's (one barrier per sub-batch)
-        if (threadIdx.x == 0) s_abort[b] = exact ? 0u : ld_volatile(a.tile_done + sg.t);
-        const int done = __syncthreads_count(s.term || !inside);
+        // thread 0 writes sub-batch j + 1's
+        if (tid == 0) s_abort[b] = exact ? 0u : ld_volatile(a.tile_done + sg.t);
+        const int ended = __syncthreads_and(q.y == kInf);
         abort = s_abort[b] != 0;
-        if (done == kRasterThreads || abort) {
+        if (ended || abort) {
             if (more) {  // drain the copies already issued
                 wait_batch(a, &bar[b ^ 1u], (par >> (b ^ 1u)) & 1u);
                 par ^= 1u << (b ^ 1u);
@@ -443,6 +588,7 @@ __device__ __forceinline__ int run_segment(const RasterArgs &a, const Seg &sg, u
             break;
         }
     }
+    if (active) s = {q.C0, q.C1, q.C2, q.T, q.last, q.evals, q.y == kInf};
     return abort ? kAborted : kWalked;
 }
 
@@ -455,12 +601,12 @@ raster_kernel(RasterArgs a) {
     __shared__ uint32_t s_wait;
     __shared__ uint32_t s_abort[2];
     if (a.use_list && *a.use_list) return;  // the list kernel blends this frame
-    float4 *aos = reinterpret_cast<float4 *>(smem);
-    WarpPairs &wp = reinterpret_cast<WarpPairs *>(smem + 2 * kBufBytes)[threadIdx.x >> 5];
     const int tid = threadIdx.x;
+    if (tid < kRecBytes / 4)  // the padding record: no power reaches its threshold
+        reinterpret_cast<float *>(smem + 2 * kBufBytes)[tid] = tid == 9 ? kInf : 0.0f;
     if (tid == 0) {
-        mbar_init(&bar[0], 1);
-        mbar_init(&bar[1], 1);
+        mbar_init(&bar[0], kChunk);
+        mbar_init(&bar[1], kChunk);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
@@ -506,20 +652,19 @@ raster_kernel(RasterArgs a) {
             exact = s_flag == kPre;
         }
         const int tx = sg.t % a.tiles_x, ty = sg.t / a.tiles_x;
-        // each warp covers an 8x4 pixel block (2 x 4 blocks per tile): close
-        // pixels accept and terminate alike, which keeps lanes converged
+        // each warp covers an 8x4 pixel block (2 x 4 blocks per tile), each
+        // half of it a 4x4 one: close pixels accept and terminate alike
         const int wid = tid >> 5, lid = tid & 31;
-        const int px = tx * 16 + (wid & 1) * 8 + (lid & 7);
-        const int py = ty * 16 + (wid >> 1) * 4 + (lid >> 3);
+        const int lx = (wid & 1) * 8 + (lid >> 4) * 4 + (lid & 3);
+        const int ly = (wid >> 1) * 4 + ((lid >> 2) & 3);
+        const int slot = fwd_index(lx, ly);
+        const int px = tx * 16 + lx, py = ty * 16 + ly;
         const bool inside = px < a.W && py < a.H;
         const float fx = (float)px + 0.5f, fy = (float)py + 0.5f;
-        // centre of the warp's block of pixel centres
-        const float cx = (float)(tx * 16 + (wid & 1) * 8) + 4.0f;
-        const float cy = (float)(ty * 16 + (wid >> 1) * 4) + 2.0f;
         PixelState s = {0.0f, 0.0f, 0.0f, 1.0f, 0u, sg.k * L, false};
         bool was_term = false;  // terminated in an earlier segment (already written)
         if (sg.k > 0 && exact) {
-            s = load_state(a.pre, a.pre2, prev);
+            s = load_state(a.pre, a.pre2, prev, slot);
             was_term = s.term;
         }
         // pass 0 walks the segment (exact from the predecessor's prefix, or
@@ -528,8 +673,8 @@ raster_kernel(RasterArgs a) {
         bool active = inside, skip = false, redone = false;
         const bool last_seg = sg.k + 1 == sg.nk;
         for (int pass = 0; pass < 2; pass++) {
-            const int rc = run_segment(a, sg, L, exact || pass == 1, active, fx, fy, cx, cy, s,
-                                       aos, wp, bar, parity, s_abort);
+            const int rc = run_segment(a, sg, L, exact || pass == 1, active, fx, fy, tx, ty, s,
+                                       smem, bar, parity, s_abort);
             if (rc == kAborted) {
                 skip = true;  // an earlier segment finished the tile
                 break;
@@ -541,7 +686,7 @@ raster_kernel(RasterArgs a) {
                 // publish the local aggregate, then look back: the nearest
                 // predecessor with a published prefix, and the aggregates
                 // after it
-                store_state(a.agg, a.agg2, c, s);
+                store_state(a.agg, a.agg2, c, slot, s);
                 __threadfence();
                 __syncthreads();
                 if (tid == 0) {
@@ -589,23 +734,23 @@ raster_kernel(RasterArgs a) {
                     break;
                 }
                 const uint32_t j = s_next;
-                in = load_state(a.pre, a.pre2, j);
+                in = load_state(a.pre, a.pre2, j, slot);
                 // fold the aggregates after j, four loads in flight at a time;
                 // stop once every pixel is known to have terminated before this
                 // segment (the segments it terminated in write it)
                 uint32_t i = j + 1;
                 for (; i + 4 <= c; i += 4) {
-                    PixelState x0 = load_state(a.agg, a.agg2, i);
-                    PixelState x1 = load_state(a.agg, a.agg2, i + 1);
-                    PixelState x2 = load_state(a.agg, a.agg2, i + 2);
-                    PixelState x3 = load_state(a.agg, a.agg2, i + 3);
+                    PixelState x0 = load_state(a.agg, a.agg2, i, slot);
+                    PixelState x1 = load_state(a.agg, a.agg2, i + 1, slot);
+                    PixelState x2 = load_state(a.agg, a.agg2, i + 2, slot);
+                    PixelState x3 = load_state(a.agg, a.agg2, i + 3, slot);
                     in = fold(fold(fold(fold(in, x0), x1), x2), x3);
                     if (__syncthreads_and(in.term || !inside)) {
                         i = c;
                         break;
                     }
                 }
-                for (; i < c; i++) in = fold(in, load_state(a.agg, a.agg2, i));
+                for (; i < c; i++) in = fold(in, load_state(a.agg, a.agg2, i, slot));
                 if (in.term) {
                     s = in;
                     was_term = true;
@@ -622,7 +767,7 @@ raster_kernel(RasterArgs a) {
             // successor ever waits for one
             const bool all_done = __syncthreads_and(s.term || !inside);
             if (!last_seg) {
-                if (!all_done) store_state(a.pre, a.pre2, c, s);
+                if (!all_done) store_state(a.pre, a.pre2, c, slot, s);
                 __threadfence();
                 __syncthreads();
                 if (tid == 0) st_release(all_done ? a.tile_done + sg.t : a.flags + c,
