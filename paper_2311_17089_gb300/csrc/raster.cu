@@ -173,25 +173,40 @@ segment_offsets_kernel(const uint32_t *__restrict__ ranges, int tiles, uint32_t 
                        uint32_t list_mean_max) {
     __shared__ uint32_t s_warp[32];
     __shared__ unsigned long long s_total;
+    pdl_wait<false>();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    for (uint32_t i = tid; i < n_zero16; i += 1024) zero[i] = make_uint4(0u, 0u, 0u, 0u);
     const int per = (tiles + 1023) / 1024;
     const int t0 = tid * per;
+    // the thread's list lengths, the first kKeep of them read once (frames
+    // of up to 8192 tiles); the ranges are read beside the zeroing's stores
+    constexpr int kKeep = 8;
+    uint32_t keep[kKeep];
+#pragma unroll
+    for (int k = 0; k < kKeep; k++) {
+        const int t = t0 + k;
+        keep[k] = k < per && t < tiles ? ranges[2 * t + 1] - ranges[2 * t] : 0u;
+    }
+    auto rest = [&](int t) { return ranges[2 * t + 1] - ranges[2 * t]; };
+    const int t1 = min(tiles, t0 + per);
+    for (uint32_t i = tid; i < n_zero16; i += 1024) zero[i] = make_uint4(0u, 0u, 0u, 0u);
     if (tid == 0) s_total = 0;
     __syncthreads();
     unsigned long long d = 0;
-    for (int t = t0; t < t0 + per && t < tiles; t++) d += ranges[2 * t + 1] - ranges[2 * t];
+#pragma unroll
+    for (int k = 0; k < kKeep; k++) d += keep[k];
+    for (int t = t0 + kKeep; t < t1; t++) d += rest(t);
     for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
     if (lane == 0 && d) atomicAdd(&s_total, d);
     __syncthreads();
     unsigned long long share = (s_total + resident - 1) / (resident > 0 ? resident : 1);
     uint32_t L = (uint32_t)(((share + kChunk - 1) / kChunk) * kChunk);
     if (L < kMinSegment) L = kMinSegment;
+    auto segs = [&](uint32_t len) { return len > L ? (len + L - 1) / L : 1u; };
     uint32_t sum = 0;
-    for (int t = t0; t < t0 + per && t < tiles; t++) {
-        uint32_t len = ranges[2 * t + 1] - ranges[2 * t];
-        sum += len > 0 ? (len + L - 1) / L : 1u;
-    }
+#pragma unroll
+    for (int k = 0; k < kKeep; k++)
+        if (t0 + k < t1) sum += segs(keep[k]);
+    for (int t = t0 + kKeep; t < t1; t++) sum += segs(rest(t));
     uint32_t x = sum;
     for (int o = 1; o < 32; o <<= 1) {
         uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
@@ -209,11 +224,17 @@ segment_offsets_kernel(const uint32_t *__restrict__ ranges, int tiles, uint32_t 
     }
     __syncthreads();
     uint32_t run = x - sum + (warp > 0 ? s_warp[warp - 1] : 0u);
-    for (int t = t0; t < t0 + per && t < tiles; t++) {
+#pragma unroll
+    for (int k = 0; k < kKeep; k++)
+        if (t0 + k < t1) {
+            off[t0 + k] = run;
+            run += segs(keep[k]);
+        }
+    for (int t = t0 + kKeep; t < t1; t++) {
         off[t] = run;
-        uint32_t len = ranges[2 * t + 1] - ranges[2 * t];
-        run += len > 0 ? (len + L - 1) / L : 1u;
+        run += segs(rest(t));
     }
+    pdl_next();
     if (tid == 1023) {
         off[tiles] = run;
         seg_len[0] = L;
@@ -600,6 +621,7 @@ raster_kernel(RasterArgs a) {
     __shared__ uint32_t s_flag;
     __shared__ uint32_t s_wait;
     __shared__ uint32_t s_abort[2];
+    pdl_wait();
     if (a.use_list && *a.use_list) return;  // the list kernel blends this frame
     const int tid = threadIdx.x;
     if (tid < kRecBytes / 4)  // the padding record: no power reaches its threshold
@@ -914,10 +936,13 @@ extern "C" int ms_raster_ex2(const ms_proj_t *proj, const ms_bins_t *bins,
     // the segmentation is the same for both kernels: the backward walks it
     // the tile kernel's ticket, flags and tile marks are zeroed by the first
     // kernel (the workspace and zero_bytes are 256-byte aligned)
-    segment_offsets_kernel<<<1, 1024, 0, st>>>(bins->ranges, (int)tiles, (uint32_t)resident,
-                                               a.seg_off, a.seg_len, reinterpret_cast<uint4 *>(w),
-                                               list ? 0u : (uint32_t)(L.zero_bytes / 16),
-                                               use_list, kListMeanMin, kListMeanMax);
+    if ((rc = cuda_check(launch_after(segment_offsets_kernel, 1, 1024, 0, st, bins->ranges, (int)tiles,
+                                      (uint32_t)resident, a.seg_off, a.seg_len,
+                                      reinterpret_cast<uint4 *>(w),
+                                      list ? 0u : (uint32_t)(L.zero_bytes / 16), use_list,
+                                      kListMeanMin, kListMeanMax),
+                         "segment offsets launch")))
+        return rc;
     if (list || band) {
         ListArgs la;
         la.ranges = a.ranges;
@@ -942,13 +967,12 @@ extern "C" int ms_raster_ex2(const ms_proj_t *proj, const ms_bins_t *bins,
         la.use_list = use_list;
         la.max_segs = (uint32_t)L.max_segs;
         la.err = a.err;
-        if ((rc = cuda_check(cudaGetLastError(), "segment offsets launch"))) return rc;
         if (group > 0) return cuda_check(launch_raster_group(la, group, st), "raster group launch");
         if ((rc = cuda_check(launch_raster_list(la, st), "raster list launch"))) return rc;
         if (!band) return MS_OK;
     }
-    raster_kernel<<<resident, kRasterThreads, kSmemBytes, st>>>(a);
-    return cuda_check(cudaGetLastError(), "raster launches");
+    return cuda_check(launch_after(raster_kernel, resident, kRasterThreads, kSmemBytes, st, a),
+                      "raster launch");
 }
 
 extern "C" int ms_raster_ex(const ms_proj_t *proj, const ms_bins_t *bins,

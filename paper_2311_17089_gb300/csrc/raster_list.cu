@@ -131,6 +131,7 @@ __device__ __forceinline__ uint32_t row_mask_of(const ListArgs &a, uint32_t g, i
 // each), so long lists are spread over many CTAs.  A frame the tile kernel
 // blends (*a.use_list == 0) is skipped.
 __global__ void __launch_bounds__(256) row_mask_kernel(ListArgs a) {
+    pdl_wait<false>();
     const uint32_t c = blockIdx.x;
     if (a.use_list && *a.use_list == 0u) return;
     if (c >= a.seg_off[a.tiles]) return;
@@ -329,6 +330,7 @@ __device__ __forceinline__ int pack_window(const ListArgs &a, uint32_t b, uint32
 // before this one is blended, and the masks and list indices of the window
 // after it are loaded while this one is blended.
 __global__ void __launch_bounds__(256, 4) raster_list_kernel(ListArgs a) {
+    pdl_wait();
     extern __shared__ __align__(16) unsigned char list_smem[];
     float4 *stage = reinterpret_cast<float4 *>(list_smem);
     uint16_t *soff = reinterpret_cast<uint16_t *>(list_smem + kPosOff);
@@ -418,10 +420,10 @@ __global__ void __launch_bounds__(256, 4) raster_list_kernel(ListArgs a) {
 cudaError_t launch_raster_list(const ListArgs &a, cudaStream_t st) {
     if (ensure_smem_attr(reinterpret_cast<const void *>(raster_list_kernel), kListSmem))
         return cudaErrorInvalidValue;
-    row_mask_kernel<<<(unsigned)a.max_segs, 256, 0, st>>>(a);
+    const cudaError_t e = launch_after(row_mask_kernel, (unsigned)a.max_segs, 256, 0, st, a);
+    if (e != cudaSuccess) return e;
     const int64_t grid = (int64_t)a.tiles * kListCtasPerTile;
-    raster_list_kernel<<<(unsigned)grid, 256, kListSmem, st>>>(a);
-    return cudaGetLastError();
+    return launch_after(raster_list_kernel, (unsigned)grid, 256, kListSmem, st, a);
 }
 
 }  // namespace msgs
