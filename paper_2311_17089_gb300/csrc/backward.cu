@@ -14,10 +14,11 @@
 //   dC/dalpha_k = T_k c_k - R_k / (1 - alpha_k),  dC/dc_k = alpha_k T_k.
 // alpha = sigma e^power (below the 0.99 clamp) gives dsigma and dpower, and
 // power = -(a dx^2 + c dy^2)/2 - b dx dy gives the centre and conic
-// gradients.  Per record, a warp reduce-scatters its 32 pixels' nine values
-// (12 shuffles; nine lanes end up owning one full sum each), the owners add
-// them to shared memory, and the CTA adds each record's sums to the
-// per-Gaussian 2D gradient with one atomic per value.
+// gradients.  The nine sums over pixels of a record are moments of dL/dpower
+// about its centre and the weights against dL/dC, so a warp keeps dL/dpower
+// and the weight of its 64 pixels for 16 records in shared memory and then
+// sums them with a record per lane (two lanes a record); the CTA adds each
+// record's sums to the per-Gaussian 2D gradient with one atomic per value.
 //
 // project_bwd_kernel: per Gaussian, the chain rule from (centre, conic,
 // opacity, colour) through V' = V + 0.3 I, V = J W Sigma W^T J^T, the
@@ -34,11 +35,12 @@
 #include "common.cuh"
 #include "f32x2.cuh"
 #include "raster_ws.cuh"
+#include "tma.cuh"
 
 namespace msgs {
 
 constexpr int kBwdThreads = 128;  // two pixels per thread
-constexpr int kBwdBatch = 256;
+constexpr int kBwdBatch = 96;  // 54 KB of shared memory: 4 CTAs per SM
 constexpr int kG2 = 9;  // dux, duy, da, db, dc, dsigma, dr, dg, db
 constexpr float kInvConicA = -1.3862943611198906f;  // 1 / (-log2(e)/2)
 constexpr float kInvConicB = -0.6931471805599453f;  // 1 / (-log2(e))
@@ -72,72 +74,147 @@ struct BwdArgs {
     uint32_t *ticket;
 };
 
-// Sum of v[q] over the 32 lanes of a warp, reduce-scattered: lane l returns
-// the full sum of value q(l) = l < 4 ? l / 2 : l / 4 + 1 when it is an
-// owner (l < 4 ? l even : l % 4 == 0), a partial sum otherwise.  Halving
-// the set of values a lane carries at every step costs 5 + 3 + 2 + 1 + 1
-// shuffles instead of 9 x 5.
-__device__ __forceinline__ float reduce_scatter9(const float v[kG2], int lane) {
-    const bool b4 = lane & 16, b3 = lane & 8, b2 = lane & 4, b1 = lane & 2;
-    // xor 16: lanes 0-15 keep values 0-4, lanes 16-31 values 5-8
-    float a[5];
-#pragma unroll
-    for (int k = 0; k < 5; k++) {
-        const float hi = k < 4 ? v[5 + k] : 0.0f;
-        const float keep = b4 ? hi : v[k], send = b4 ? v[k] : hi;
-        a[k] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
-    }
-    // xor 8: {0,1,2 | 3,4} and {5,6 | 7,8}
-    float b[3];
-#pragma unroll
-    for (int k = 0; k < 3; k++) {
-        const float hi = b4 ? (k + 2 < 5 ? a[k + 2] : 0.0f) : (k + 3 < 5 ? a[k + 3] : 0.0f);
-        const float keep = b3 ? hi : a[k], send = b3 ? a[k] : hi;
-        b[k] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
-    }
-    // xor 4: {0,1 | 2}, {3 | 4}, {5 | 6}, {7 | 8}
-    const bool g3 = !b4 && !b3;
-    float c[2];
-#pragma unroll
-    for (int k = 0; k < 2; k++) {
-        const float hi = g3 ? (k + 2 < 3 ? b[k + 2] : 0.0f) : b[k + 1];
-        const float keep = b2 ? hi : b[k], send = b2 ? b[k] : hi;
-        c[k] = keep + __shfl_xor_sync(0xffffffffu, send, 4);
-    }
-    // xor 2: {0 | 1}; every other group holds one value
-    const bool two = g3 && !b2;
-    const float keep = (two && b1) ? c[1] : c[0];
-    const float send = two ? (b1 ? c[0] : c[1]) : c[0];
-    const float d = keep + __shfl_xor_sync(0xffffffffu, send, 2);
-    return d + __shfl_xor_sync(0xffffffffu, d, 1);
-}
-
-// Two pixels of one thread, (x, y) and (x, y + 4): the same dx for every
-// record, so their arithmetic runs as packed FP32x2 pairs.
+// A thread takes two pixels, (x, y) and (x, y + 4) of its warp's 8x8 block,
+// as packed FP32x2 pairs: T, the colour still behind weighted by dL/dC, R =
+// sum_c dL/dC_c (C_c - F_c), and dL/dC.  With g = sum_c dL/dC_c c_k,c of
+// record k, R_k = R_{k-1} - w_k g and dL/dalpha_k = T_k g - R_k / (1 - alpha_k).
 struct PixPair {
-    f32x2 T, F0, F1, F2, C0, C1, C2, d0, d1, d2;
-    uint32_t cntA, cntB;  // entries of the segment each pixel blended through
+    f32x2 T, R, d0, d1, d2;
+    int cntA, cntB;  // entries of the segment each pixel blended through
 };
 
-__global__ void __launch_bounds__(kBwdThreads, 8)  // 64 registers: 8 CTAs per SM
+// Per warp: for kBwdSlots records and the block's 64 pixels (row by row)
+// dL/dpower and the weight w, a pixel's row kBwdSlots + 1 floats long, the
+// second 32 pixels a half bank row further (the warp's halves read them at
+// once); the pixels' dL/dC.
+constexpr int kBwdSlots = 16;
+constexpr int kRowF = kBwdSlots + 1;
+constexpr int kHalfF = 32 * kRowF + 16;
+struct BwdWarp {
+    float4 d[64];
+    float q[2 * kHalfF - 16], w[2 * kHalfF - 16];
+    uint16_t list[kBwdBatch];  // records in reach
+    uint16_t slot[kBwdSlots];  // the slots' records
+};
+struct BwdSmem {
+    BwdWarp warp[kBwdThreads / 32];
+    float4 rec[2][kBwdBatch * 3];
+    uint32_t idx[2][kBwdBatch];
+    float acc[kBwdBatch][kG2 + 1];  // [kG2] marks a record some pixel took
+};
+
+// The record's alpha can reach 1/255 at some pixel centre of the 8x8 block
+// centred on (cx, cy): its level-set box reaches the block, and so does the
+// level set itself (power log2(e) = A dx^2 + B dx dy + C dy^2 is concave, so
+// over a rectangle that does not hold the centre its maximum lies on the
+// side nearest in x or the one nearest in y, at a clamped division).  The
+// margin covers the rounding of this evaluation and of the pixels', each a
+// few 2^-24 of the terms' magnitudes; NaN keeps the record.
+__device__ __forceinline__ bool reaches_block(const float4 r0, float C, const float4 r2, float cx,
+                                              float cy) {
+    constexpr float kHalf = 3.5f, kReach = 3.5625f;
+    if (!(fabsf(r0.x - cx) <= r2.z + kReach && fabsf(r0.y - cy) <= r2.w + kReach)) return false;
+    const float A = r0.z, B = r0.w;
+    const float xl = cx - kHalf - r0.x, xh = cx + kHalf - r0.x;
+    const float yl = cy - kHalf - r0.y, yh = cy + kHalf - r0.y;
+    const float xn = fmaxf(xl, fminf(0.0f, xh)), yn = fmaxf(yl, fminf(0.0f, yh));
+    const float ys = fminf(yh, fmaxf(yl, -0.5f * B * __fdividef(xn, C)));
+    const float xs = fminf(xh, fmaxf(xl, -0.5f * B * __fdividef(yn, A)));
+    const float p1 = (A * xn + B * ys) * xn + C * ys * ys;
+    const float p2 = (A * xs + B * yn) * xs + C * yn * yn;
+    const float X = fmaxf(fabsf(xl), fabsf(xh)), Y = fmaxf(fabsf(yl), fabsf(yh));
+    const float m = 1.52587890625e-5f * (fabsf(A) * X * X + fabsf(B) * X * Y + fabsf(C) * Y * Y);
+    return !(fmaxf(p1, p2) < r2.y - m);
+}
+
+// The nine sums of the warp's first n slots, a record per lane pair (lane
+// and lane + 16 take 32 pixels each): the pixels' weights against dL/dC, and
+// the moments of dL/dpower about the block's centre (bcx, bcy), shifted to
+// the record's.  Added to the CTA's sums.
+__device__ __forceinline__ void add_slots(const BwdWarp &wp, uint32_t n, const float4 *rec,
+                                          float bcx, float bcy, float (*acc)[kG2 + 1]) {
+    const uint32_t lane = threadIdx.x & 31u, r = lane & 15u, h = lane >> 4;
+    const float *q = wp.q + h * kHalfF + r, *w = wp.w + h * kHalfF + r;
+    const float4 *d = wp.d + 32 * h;
+    float m0 = 0.0f, mx = 0.0f, my = 0.0f, mxx = 0.0f, mxy = 0.0f, myy = 0.0f;
+    float w0 = 0.0f, w1 = 0.0f, w2 = 0.0f;
+    const float y0 = h ? 0.5f : -3.5f;
+#pragma unroll
+    for (int row = 0; row < 4; row++) {
+        float r0 = 0.0f, r1 = 0.0f, r2 = 0.0f;
+#pragma unroll
+        for (int x = 0; x < 8; x++) {
+            const int p = row * 8 + x;
+            const float X = (float)x - 3.5f;
+            const float qv = q[p * kRowF], wv = w[p * kRowF];
+            const float4 dv = d[p];
+            r0 += qv;
+            r1 = fmaf(qv, X, r1);
+            r2 = fmaf(qv, X * X, r2);
+            w0 = fmaf(wv, dv.x, w0);
+            w1 = fmaf(wv, dv.y, w1);
+            w2 = fmaf(wv, dv.z, w2);
+        }
+        const float Y = y0 + (float)row;
+        m0 += r0;
+        mx += r1;
+        mxx += r2;
+        my = fmaf(Y, r0, my);
+        mxy = fmaf(Y, r1, mxy);
+        myy = fmaf(Y * Y, r0, myy);
+    }
+    float v[kG2] = {m0, mx, my, mxx, mxy, myy, w0, w1, w2};
+#pragma unroll
+    for (int k = 0; k < kG2; k++) v[k] += __shfl_xor_sync(0xffffffffu, v[k], 16);
+    if (r >= n) return;
+    const uint32_t j = wp.slot[r];
+    const float4 r0 = rec[3 * j];
+    const float2 r1 = *reinterpret_cast<const float2 *>(rec + 3 * j + 1);
+    const float dx = bcx - r0.x, dy = bcy - r0.y;
+    const float Dx = fmaf(dx, v[0], v[1]), Dy = fmaf(dy, v[0], v[2]);
+    const float ca = r0.z * kInvConicA, cb = r0.w * kInvConicB, cc = r1.x * kInvConicA;
+    // the first lane of a pair adds the centre and conic sums, the second
+    // the opacity and colours
+    if (h == 0) {
+        atomicAdd(&acc[j][0], ca * Dx + cb * Dy);
+        atomicAdd(&acc[j][1], cb * Dx + cc * Dy);
+        atomicAdd(&acc[j][2], -0.5f * fmaf(dx, Dx + v[1], v[3]));
+        atomicAdd(&acc[j][3], -(v[4] + dx * v[2] + dy * Dx));
+        atomicAdd(&acc[j][4], -0.5f * fmaf(dy, Dy + v[2], v[5]));
+        acc[j][kG2] = 1.0f;
+    } else {
+        atomicAdd(&acc[j][5], v[0] / r1.y);
+        atomicAdd(&acc[j][6], v[6]);
+        atomicAdd(&acc[j][7], v[7]);
+        atomicAdd(&acc[j][8], v[8]);
+    }
+}
+
+// Bound by instruction issue.  A record costs a warp about 55 instructions
+// for its 64 pixels' gradients and 24 for the nine sums over them: those are
+// 9 x 64 products with per-pixel factors, formed 16 records at a time with a
+// record per lane, instead of nine reductions across the warp per record
+// (12 shuffles and about 70 instructions).  With the per-pixel state cut from
+// three colours to their product with dL/dC, records culled by their level
+// set instead of its box, and cp.async staging: the 4-view batch of 1M
+// Gaussians (1256x832, 314x208, 78x52, 19x13) 825 -> 606 us.
+__global__ void __launch_bounds__(kBwdThreads, 4)
 raster_bwd_kernel(const __grid_constant__ BwdArgs args) {
-    __shared__ float4 s_r0[kBwdBatch], s_r1[kBwdBatch];
-    __shared__ float4 s_r2[kBwdBatch];             // b, thr, ex, ey
-    __shared__ uint32_t s_idx[kBwdBatch];
-    __shared__ uint16_t s_list[kBwdThreads / 32][kBwdBatch];  // per warp: records in reach
-    __shared__ float s_acc[kBwdBatch][kG2 + 1];  // [kG2] marks a record some pixel took
+    pdl_wait();
+    extern __shared__ __align__(128) unsigned char bwd_smem[];
+    BwdSmem &sm = *reinterpret_cast<BwdSmem *>(bwd_smem);
     __shared__ uint32_t s_c, s_cnt;
     __shared__ uint32_t s_first[kMaxViews + 1];   // first ticket of each view's segments
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    const bool owner = lane < 4 ? (lane & 1) == 0 : (lane & 3) == 0;
-    const int q_own = lane < 4 ? lane >> 1 : (lane >> 2) + 1;
+    BwdWarp &wp = sm.warp[wid];
     // this thread's pixels within a tile: warp w covers the 8x8 block
     // ((w & 1) * 8, (w >> 1) * 8), lane l the pixels (l & 7, l >> 3) and
     // (l & 7, (l >> 3) + 4) of it
     const int lx = (wid & 1) * 8 + (lane & 7);
     const int lyA = (wid >> 1) * 8 + (lane >> 3), lyB = lyA + 4;
     const int fA = fwd_index(lx, lyA), fB = fwd_index(lx, lyB);
-    for (int i = tid; i < kBwdBatch * (kG2 + 1); i += kBwdThreads) (&s_acc[0][0])[i] = 0.0f;
+    for (int i = tid; i < kBwdBatch * (kG2 + 1); i += kBwdThreads) (&sm.acc[0][0])[i] = 0.0f;
+    for (int i = lane; i < (int)(sizeof(wp.q) / 4); i += 32) wp.q[i] = wp.w[i] = 0.0f;
     if (tid == 0) {
         uint32_t run = 0;
         for (int k = 0; k < args.n_views; k++) {
@@ -164,13 +241,15 @@ raster_bwd_kernel(const __grid_constant__ BwdArgs args) {
         const uint32_t c = cg - s_first[view];
         const uint32_t L = a.seg_len[0];
         // the segment: tile t, index k within the tile, list entries [start, start + len)
-        int lo = 0, hi = a.tiles;
-        while (hi - lo > 1) {
-            const int mid = (lo + hi) >> 1;
-            if (a.seg_off[mid] <= c) lo = mid;
-            else hi = mid;
+        uint32_t lo = 0, hi = (uint32_t)a.tiles;
+        while (hi - lo > 1u) {  // the warp's lanes search together
+            const uint32_t step = (hi - lo + 31u) / 32u, q = lo + (lane + 1u) * step;
+            const uint32_t n =
+                __popc(__ballot_sync(0xffffffffu, q < hi && __ldg(a.seg_off + q) <= c));
+            lo += n * step;
+            hi = min(hi, lo + step);
         }
-        const int t = lo;
+        const int t = (int)lo;
         const uint32_t k = c - a.seg_off[t];
         const uint32_t tbeg = a.ranges[2 * t], tend = a.ranges[2 * t + 1];
         const uint32_t pos0 = k * L;  // tile-relative position of the first entry
@@ -179,91 +258,89 @@ raster_bwd_kernel(const __grid_constant__ BwdArgs args) {
         const int tx = t % a.tiles_x, ty = t / a.tiles_x;
         const int px = tx * 16 + lx;
         PixPair pp;
-        float st[2][10];  // per pixel: T, F0..2, C0..2, d0..2
+        float st[2][5];  // per pixel: T, R, d0..2
         uint32_t cnt[2] = {0u, 0u};
 #pragma unroll
         for (int h = 0; h < 2; h++) {
             const int py = ty * 16 + (h ? lyB : lyA);
             st[h][0] = 1.0f;
 #pragma unroll
-            for (int q = 1; q < 10; q++) st[h][q] = 0.0f;
+            for (int q = 1; q < 5; q++) st[h][q] = 0.0f;
             if (px < a.W && py < a.H && len > 0) {
                 const size_t p = (size_t)py * a.W + px, plane = (size_t)a.W * a.H;
                 const uint32_t nc = a.n_contrib[p];
                 if (nc > pos0) {
                     cnt[h] = min(nc - pos0, len);
-                    if (k > 0) {
-                        const float4 s4 =
-                            __ldcg(a.pre + (size_t)(c - 1) * kRasterThreads + (h ? fB : fA));
-                        st[h][0] = s4.w;
-                        st[h][1] = s4.x;
-                        st[h][2] = s4.y;
-                        st[h][3] = s4.z;
-                    }
-                    st[h][4] = a.image[p];
-                    st[h][5] = a.image[plane + p];
-                    st[h][6] = a.image[2 * plane + p];
-                    st[h][7] = a.dl[p];
-                    st[h][8] = a.dl[plane + p];
-                    st[h][9] = a.dl[2 * plane + p];
+                    float4 s4 = make_float4(0.0f, 0.0f, 0.0f, 1.0f);
+                    if (k > 0)
+                        s4 = __ldcg(a.pre + (size_t)(c - 1) * kRasterThreads + (h ? fB : fA));
+                    const float d0 = a.dl[p], d1 = a.dl[plane + p], d2 = a.dl[2 * plane + p];
+                    st[h][0] = s4.w;
+                    st[h][1] = d0 * (a.image[p] - s4.x) + d1 * (a.image[plane + p] - s4.y) +
+                               d2 * (a.image[2 * plane + p] - s4.z);
+                    st[h][2] = d0;
+                    st[h][3] = d1;
+                    st[h][4] = d2;
                 }
             }
+            wp.d[lane + 32 * h] = make_float4(st[h][2], st[h][3], st[h][4], 0.0f);
         }
         pp.T = pack2(st[0][0], st[1][0]);
-        pp.F0 = pack2(st[0][1], st[1][1]);
-        pp.F1 = pack2(st[0][2], st[1][2]);
-        pp.F2 = pack2(st[0][3], st[1][3]);
-        pp.C0 = pack2(st[0][4], st[1][4]);
-        pp.C1 = pack2(st[0][5], st[1][5]);
-        pp.C2 = pack2(st[0][6], st[1][6]);
-        pp.d0 = pack2(st[0][7], st[1][7]);
-        pp.d1 = pack2(st[0][8], st[1][8]);
-        pp.d2 = pack2(st[0][9], st[1][9]);
-        pp.cntA = cnt[0];
-        pp.cntB = cnt[1];
+        pp.R = pack2(st[0][1], st[1][1]);
+        pp.d0 = pack2(st[0][2], st[1][2]);
+        pp.d1 = pack2(st[0][3], st[1][3]);
+        pp.d2 = pack2(st[0][4], st[1][4]);
+        pp.cntA = (int)cnt[0];
+        pp.cntB = (int)cnt[1];
         const float fx = (float)px + 0.5f;
         const f32x2 fy2 = pack2((float)(ty * 16 + lyA) + 0.5f, (float)(ty * 16 + lyB) + 0.5f);
         // centre of the warp's 8x8 block of pixel centres
         const float bcx = (float)(tx * 16 + (wid & 1) * 8) + 4.0f;
         const float bcy = (float)(ty * 16 + (wid >> 1) * 8) + 4.0f;
-        const uint32_t wcnt = __reduce_max_sync(0xffffffffu, max(pp.cntA, pp.cntB));
+        const uint32_t wcnt = __reduce_max_sync(0xffffffffu, max(cnt[0], cnt[1]));
         if (lane == 0 && wcnt) atomicMax(&s_cnt, wcnt);
         __syncthreads();
         const uint32_t cnt_seg = s_cnt;
-        for (uint32_t off = 0; off < cnt_seg; off += kBwdBatch) {
-            const uint32_t nb = min(cnt_seg - off, (uint32_t)kBwdBatch);
-            for (uint32_t r = tid; r < nb; r += kBwdThreads) {
-                uint32_t g = a.gidx[start + off + r];
+        // stage one batch of records: a record per thread
+        auto stage = [&](uint32_t off, uint32_t b) {
+            if (tid < kBwdBatch && off + tid < cnt_seg) {
+                uint32_t g = a.gidx[start + off + tid];
                 if (g >= a.n_rec) g = 0;  // unreachable unless binning reported an error
-                s_idx[r] = g;
-                s_r0[r] = a.rec[3 * (size_t)g];
-                s_r1[r] = a.rec[3 * (size_t)g + 1];
-                s_r2[r] = a.rec[3 * (size_t)g + 2];
+                sm.idx[b][tid] = g;
+                const float4 *src = a.rec + 3 * (size_t)g;
+                float4 *dst = sm.rec[b] + 3 * tid;
+                cp_async16(dst, src);
+                cp_async16(dst + 1, src + 1);
+                cp_async16(dst + 2, src + 2);
             }
-            __syncthreads();
+            cp_async_commit();
+        };
+        if (cnt_seg) stage(0u, 0u);
+        for (uint32_t off = 0, b = 0; off < cnt_seg; off += kBwdBatch, b ^= 1u) {
+            const uint32_t nb = min(cnt_seg - off, (uint32_t)kBwdBatch);
+            cp_async_wait<0>();
+            __syncthreads();  // also: the other buffer and the sums are free
+            if (off + kBwdBatch < cnt_seg) stage(off + kBwdBatch, b ^ 1u);
+            const float4 *rec = sm.rec[b];
             const uint32_t jn = wcnt > off ? min(wcnt - off, nb) : 0u;  // warp-uniform
-            // the records whose level-set box reaches the warp's
-            // 8x8 block of pixel centres, in list order; any other record has
-            // alpha < 1/255 at all of the warp's pixels
+            // the records that can reach the warp's block, in list order; any
+            // other has alpha < 1/255 at all of the warp's pixels
             uint32_t nl = 0;
             for (uint32_t j0 = 0; j0 < jn; j0 += 32) {
                 const uint32_t j = j0 + lane;
-                bool rel = false;
-                if (j < jn) {
-                    const float4 r0 = s_r0[j], r2 = s_r2[j];
-                    // half extents of the 8x8 block of pixel centres, plus
-                    // 1/16 px for the FP32 rounding of the level-set box
-                    rel = fabsf(r0.x - bcx) <= r2.z + 3.5625f && fabsf(r0.y - bcy) <= r2.w + 3.5625f;
-                }
+                const bool rel = j < jn && reaches_block(rec[3 * j], rec[3 * j + 1].x,
+                                                         rec[3 * j + 2], bcx, bcy);
                 const uint32_t m = __ballot_sync(0xffffffffu, rel);
-                if (rel) s_list[wid][nl + __popc(m & ((1u << lane) - 1u))] = (uint16_t)j;
+                if (rel) wp.list[nl + __popc(m & ((1u << lane) - 1u))] = (uint16_t)j;
                 nl += __popc(m);
             }
             __syncwarp();
+            const int limA = pp.cntA - (int)off, limB = pp.cntB - (int)off;
+            uint32_t ns = 0;  // slots filled
             for (uint32_t li = 0; li < nl; li++) {
-                const uint32_t j = s_list[wid][li];
-                const float4 r0 = s_r0[j], r1 = s_r1[j];
-                const float4 r2 = s_r2[j];
+                const uint32_t j = wp.list[li];
+                const float4 r0 = rec[3 * j], r1 = rec[3 * j + 1];
+                const float2 r2 = *reinterpret_cast<const float2 *>(rec + 3 * j + 2);
                 // the forward's exact FP32 operations, for both pixels
                 const float dx = __fsub_rn(fx, r0.x);
                 const f32x2 dy = sub2(fy2, splat2(r0.y));
@@ -271,79 +348,55 @@ raster_bwd_kernel(const __grid_constant__ BwdArgs args) {
                 const f32x2 pw = fma2(mul2(splat2(r1.x), dy), dy, mul2(splat2(dx), u));
                 float pA, pB;
                 unpack2(pw, pA, pB);
-                const bool accA = off + j < pp.cntA && pA <= 0.0f && pA >= r2.y;
-                const bool accB = off + j < pp.cntB && pB <= 0.0f && pB >= r2.y;
+                const bool accA = (int)j < limA && pA <= 0.0f && pA >= r2.y;
+                const bool accB = (int)j < limB && pB <= 0.0f && pB >= r2.y;
                 if (!__any_sync(0xffffffffu, accA || accB)) continue;
-                // alpha of accepted pixels, 0 for the others (no effect on
-                // T, F or any gradient); gradients through alpha only below
-                // the 0.99 clamp
-                const float eA = ex2_approx_b(accA ? pA : -256.0f);
-                const float eB = ex2_approx_b(accB ? pB : -256.0f);
-                const float GA = r1.y * eA, GB = r1.y * eB;
+                // alpha of accepted pixels, 0 for the others (no effect on T,
+                // R or any gradient); gradients through alpha only below the
+                // 0.99 clamp
+                const float GA = r1.y * ex2_approx_b(accA ? pA : -256.0f);
+                const float GB = r1.y * ex2_approx_b(accB ? pB : -256.0f);
                 const float alA = accA ? fminf(0.99f, GA) : 0.0f;
                 const float alB = accB ? fminf(0.99f, GB) : 0.0f;
-                const f32x2 al = pack2(alA, alB);
-                const f32x2 mg = pack2(accA && GA < 0.99f ? 1.0f : 0.0f,
-                                       accB && GB < 0.99f ? 1.0f : 0.0f);
-                const f32x2 e = pack2(eA, eB);
+                const f32x2 al = pack2(alA, alB), nal = pack2(-alA, -alB);
+                const f32x2 ag = pack2(GA < 0.99f ? alA : 0.0f, GB < 0.99f ? alB : 0.0f);
+                const f32x2 g = fma2(splat2(r2.x), pp.d2,
+                                     fma2(splat2(r1.w), pp.d1, mul2(splat2(r1.z), pp.d0)));
                 const f32x2 w = mul2(al, pp.T);
-                const f32x2 cr = splat2(r1.z), cg2 = splat2(r1.w), cb2 = splat2(r2.x);
-                pp.F0 = fma2(w, cr, pp.F0);
-                pp.F1 = fma2(w, cg2, pp.F1);
-                pp.F2 = fma2(w, cb2, pp.F2);
-                const f32x2 om = sub2(splat2(1.0f), al);
-                const f32x2 iom = pack2(__fdividef(1.0f, 1.0f - alA), __fdividef(1.0f, 1.0f - alB));
-                // dC/dalpha = T c - (C - F) / (1 - alpha), summed over channels with dL/dC
-                const f32x2 t0 = fma2(sub2(pp.C0, pp.F0), mul2(splat2(-1.0f), iom),
-                                      mul2(pp.T, cr));
-                const f32x2 t1 = fma2(sub2(pp.C1, pp.F1), mul2(splat2(-1.0f), iom),
-                                      mul2(pp.T, cg2));
-                const f32x2 t2 = fma2(sub2(pp.C2, pp.F2), mul2(splat2(-1.0f), iom),
-                                      mul2(pp.T, cb2));
-                const f32x2 dal = fma2(pp.d2, t2, fma2(pp.d1, t1, mul2(pp.d0, t0)));
-                pp.T = mul2(pp.T, om);
-                const f32x2 hd = mul2(mul2(dal, mg), e);     // dL/dsigma terms
-                const f32x2 dpow = mul2(mul2(dal, mg), al);  // dL/dpower terms
-                const float ca = r0.z * kInvConicA, cb = r0.w * kInvConicB, cc = r1.x * kInvConicA;
-                const f32x2 gx = fma2(splat2(cb), dy, splat2(ca * dx));
-                const f32x2 gy = fma2(splat2(cc), dy, splat2(cb * dx));
-                float v[kG2], lo2, hi2;
-                unpack2(mul2(dpow, gx), lo2, hi2);
-                v[0] = lo2 + hi2;
-                unpack2(mul2(dpow, gy), lo2, hi2);
-                v[1] = lo2 + hi2;
-                unpack2(dpow, lo2, hi2);
-                v[2] = (lo2 + hi2) * (-0.5f * dx * dx);
-                unpack2(mul2(dpow, dy), lo2, hi2);
-                v[3] = -dx * (lo2 + hi2);
-                unpack2(mul2(mul2(dpow, dy), dy), lo2, hi2);
-                v[4] = -0.5f * (lo2 + hi2);
-                unpack2(hd, lo2, hi2);
-                v[5] = lo2 + hi2;
-                unpack2(mul2(w, pp.d0), lo2, hi2);
-                v[6] = lo2 + hi2;
-                unpack2(mul2(w, pp.d1), lo2, hi2);
-                v[7] = lo2 + hi2;
-                unpack2(mul2(w, pp.d2), lo2, hi2);
-                v[8] = lo2 + hi2;
-                const float sum = reduce_scatter9(v, lane);
-                if (owner) {
-                    atomicAdd(&s_acc[j][q_own], sum);
-                    if (lane == 0) s_acc[j][kG2] = 1.0f;
+                pp.R = fma2(mul2(nal, pp.T), g, pp.R);
+                const f32x2 nio = pack2(-__fdividef(1.0f, 1.0f - alA), -__fdividef(1.0f, 1.0f - alB));
+                const f32x2 dal = fma2(pp.R, nio, mul2(pp.T, g));
+                pp.T = fma2(nal, pp.T, pp.T);
+                float q0, q1, w0, w1;
+                unpack2(mul2(dal, ag), q0, q1);  // dL/dpower
+                unpack2(w, w0, w1);
+                const uint32_t at = (uint32_t)lane * kRowF + ns;
+                wp.q[at] = q0;
+                wp.q[kHalfF + at] = q1;
+                wp.w[at] = w0;
+                wp.w[kHalfF + at] = w1;
+                if (lane == 0) wp.slot[ns] = (uint16_t)j;
+                if (++ns == kBwdSlots) {
+                    __syncwarp();
+                    add_slots(wp, ns, rec, bcx, bcy, sm.acc);
+                    __syncwarp();
+                    ns = 0;
                 }
             }
+            if (ns) {
+                __syncwarp();
+                add_slots(wp, ns, rec, bcx, bcy, sm.acc);
+            }
             __syncthreads();
-            for (uint32_t r = tid; r < nb; r += kBwdThreads) {
-                if (s_acc[r][kG2] == 0.0f) continue;
-                float *dst = a.g2 + (size_t)s_idx[r] * kG2;
+            if ((uint32_t)tid < nb && sm.acc[tid][kG2] != 0.0f) {
+                float *dst = a.g2 + (size_t)sm.idx[b][tid] * kG2;
 #pragma unroll
                 for (int q = 0; q < kG2; q++) {
-                    if (s_acc[r][q] != 0.0f) atomicAdd(dst + q, s_acc[r][q]);
-                    s_acc[r][q] = 0.0f;
+                    if (sm.acc[tid][q] != 0.0f) atomicAdd(dst + q, sm.acc[tid][q]);
+                    sm.acc[tid][q] = 0.0f;
                 }
-                s_acc[r][kG2] = 0.0f;
+                sm.acc[tid][kG2] = 0.0f;
             }
-            __syncthreads();
         }
     }
 }
@@ -645,6 +698,7 @@ struct ColorRows {
 template <int DEG>
 __global__ void __launch_bounds__(kProjBwdWarps * 32)
 project_bwd_kernel(const __grid_constant__ ProjBwdArgs p) {
+    pdl_wait();
     using CR = ColorRows<DEG>;
     extern __shared__ float s_rows[];
     __shared__ CamB s_cam[kMaxViews];  // lanes on different views read them at once
@@ -721,8 +775,8 @@ static int launch_project_bwd(const ProjBwdArgs &pb, cudaStream_t st) {
     const int64_t warps = ceil_div(pb.sc.n, 32);
     const int grid = (int)std::max<int64_t>(
         1, std::min<int64_t>(ceil_div(warps, kProjBwdWarps), (int64_t)num_sms() * 16));
-    project_bwd_kernel<DEG><<<grid, kProjBwdWarps * 32, smem, st>>>(pb);
-    return MS_OK;
+    return cuda_check(launch_after(project_bwd_kernel<DEG>, grid, kProjBwdWarps * 32, smem, st, pb),
+                      "project backward launch");
 }
 
 constexpr int kL1Threads = 256;
@@ -795,8 +849,8 @@ static int raster_bwd_blocks_per_sm() {
     static std::atomic<int> v{0};
     int b = v.load(std::memory_order_relaxed);
     if (b == 0) {
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, raster_bwd_kernel, kBwdThreads, 0) !=
-                cudaSuccess ||
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, raster_bwd_kernel, kBwdThreads,
+                                                          sizeof(BwdSmem)) != cudaSuccess ||
             b < 1)
             b = 1;
         v.store(b, std::memory_order_relaxed);
@@ -887,7 +941,13 @@ extern "C" int ms_raster_bwd_views(const ms_scene_t *scene, const ms_bwd_view_t 
     if (raster_pass) {
         if ((rc = cuda_check(cudaMemsetAsync(ws, 0, need, st), "bwd workspace memset")))
             return rc;
-        raster_bwd_kernel<<<raster_bwd_blocks_per_sm() * num_sms(), kBwdThreads, 0, st>>>(a);
+        if ((rc = ensure_smem_attr(reinterpret_cast<const void *>(raster_bwd_kernel),
+                                   sizeof(BwdSmem))))
+            return rc;
+        if ((rc = cuda_check(launch_after(raster_bwd_kernel, raster_bwd_blocks_per_sm() * num_sms(),
+                                          kBwdThreads, sizeof(BwdSmem), st, a),
+                             "raster backward launch")))
+            return rc;
     }
     if (n > 0 && project_pass) {
         pb.sc.n = n;
