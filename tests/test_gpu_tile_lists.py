@@ -1,7 +1,7 @@
 """ms_bin and ms_bin_ordered on made-up projections, so that every cut of the
-tile stage is met: one tile to 65536, empty to full frames, Gaussians of one
-tile and of all of them, orders around a block's 1024 positions and past
-2048 blocks, capacities from one entry to more than needed.  The lists,
+tile stage (and the one-CTA depth sort) is met: one tile to 65536, empty to
+full frames, Gaussians of one tile and of all of them, orders around a
+block's 1024 positions and past 2048 blocks, capacities from one entry to more than needed.  The lists,
 ranges and counts equal a host reference bit for bit: the listed Gaussians
 by (depth bits, index), each one's tiles row by row, the first dup_capacity
 of these entries, stably sorted by tile."""
@@ -129,6 +129,8 @@ CASES = [
     (6000, 79, 52, "mixed"), (150, 79, 52, "all"), (2000, 96, 64, "small"), (2000, 97, 64, "small"),
     (1500, 128, 128, "mixed"), (1500, 129, 128, "mixed"), (700, 256, 256, "mixed"),
     (900, 2048, 32, "big"), (200000, 20, 13, "mixed"),
+    # around the largest projection one CTA sorts
+    (4095, 39, 27, "mixed"), (4096, 10, 7, "small"), (4096, 39, 27, "big"), (4097, 10, 7, "mixed"),
 ]
 
 
