@@ -627,9 +627,13 @@ class Renderer:
         max_ctas_per_sm caps the tile kernel's CTAs (ms_raster_ex2)."""
         if cam.tiles_x * cam.tiles_y > self.max_tiles:
             raise MsError(MS_ERR_INVALID_ARG, "camera has more tiles than max_tiles")
-        ms_project(scene.struct, camera_struct(cam), MODES.get(mode, mode), self.proj, stream)
-        return self.bin_raster(scene, cam, out, stream, n_eval, strategy,
-                               max_ctas_per_sm=max_ctas_per_sm)
+        import torch
+        # one look-up of the stream and one camera struct for the three calls
+        stream = torch.cuda.current_stream() if stream is None else stream
+        cs = camera_struct(cam)
+        ms_project(scene.struct, cs, MODES.get(mode, mode), self.proj, stream)
+        ms_bin(self.proj, scene.n, cs, self.bins, _ptr(self.ws), self.ws_bytes, stream)
+        return self._raster(cs, cam, out, stream, n_eval, strategy, max_ctas_per_sm)
 
     def bin(self, scene: DeviceScene, cam: inputs.Camera, stream=None, order=None):
         """Enqueue the binning of this renderer's projection (left by
@@ -652,7 +656,10 @@ class Renderer:
                max_ctas_per_sm=0):
         """Enqueue the blend of this renderer's bins (ms_raster_ex2).
         Returns the (image, final_t, n_contrib) device tensors."""
-        cs = camera_struct(cam)
+        return self._raster(camera_struct(cam), cam, out, stream, n_eval, strategy,
+                            max_ctas_per_sm)
+
+    def _raster(self, cs, cam, out, stream, n_eval, strategy, max_ctas_per_sm):
         image, final_t, n_contrib = out if out is not None else self.images(cam)
         ms_raster_ex2(self.proj, self.bins, cs, _ptr(image), _ptr(final_t), _ptr(n_contrib),
                       _ptr(n_eval), _ptr(self.rws), self.rws_bytes,

@@ -11,9 +11,9 @@ from __future__ import annotations
 import torch
 
 from . import (MODES, STRATEGIES, MsError, MS_OK, MS_MAX_BWD_VIEWS, Renderer, _ptr, bwd_view,
-               camera_struct, ms_bin, ms_bin_counts, ms_grads_t, ms_project, ms_raster_ex2,
+               camera_struct, ms_bin, ms_bin_counts, ms_grads_t, ms_project, ms_project_views,
                ms_raster_bwd, ms_raster_bwd_views, ms_raster_bwd_views_workspace_bytes,
-               ms_raster_bwd_workspace_bytes, ms_scene_prepare, ms_scene_t)
+               ms_raster_bwd_workspace_bytes, ms_raster_ex2, ms_scene_prepare, ms_scene_t)
 from . import inputs
 
 
@@ -113,15 +113,23 @@ class GaussianRenderViews(torch.autograd.Function):
         sc = _scene_struct(n, n_levels, sh_degree, mean, log_scale, quat, opacity, color,
                            level, s_max, s_min, scale, lnop)
         ms_scene_prepare(sc)
+        # every view's projection in one pass over the scene (frames that
+        # share buffers, one after the other)
+        cams = [camera_struct(f.cam) for f in frames]
+        stream = torch.cuda.current_stream()
+        m = MODES.get(mode, mode)
+        together = len({id(f.renderer) for f in frames}) == len(frames)
+        if together:
+            ms_project_views(sc, cams, m, [f.renderer.proj for f in frames], stream)
         outs = []
-        for frame in frames:
+        for frame, cs in zip(frames, cams):
             r = frame.renderer
-            cs = camera_struct(frame.cam)
-            ms_project(sc, cs, MODES.get(mode, mode), r.proj)
-            ms_bin(r.proj, n, cs, r.bins, _ptr(r.ws), r.ws_bytes)
+            if not together:
+                ms_project(sc, cs, m, r.proj, stream)
+            ms_bin(r.proj, n, cs, r.bins, _ptr(r.ws), r.ws_bytes, stream)
             ms_raster_ex2(r.proj, r.bins, cs, _ptr(frame.image), _ptr(frame.final_t),
                           _ptr(frame.n_contrib), 0, _ptr(r.rws), r.rws_bytes, frame.strategy,
-                          frame.max_ctas_per_sm)
+                          frame.max_ctas_per_sm, stream)
             outs.append(frame.image.clone())
         ctx.frames = frames
         ctx.meta = (n, n_levels, sh_degree)
