@@ -105,6 +105,12 @@ __device__ __forceinline__ float2 lds2(uint32_t p) {
     return v;
 }
 
+__device__ __forceinline__ uint2 lds_offsets(uint32_t p) {
+    uint2 v;
+    asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(p));
+    return v;
+}
+
 struct RasterArgs {
     const uint32_t *ranges;
     const uint32_t *gidx;
@@ -256,7 +262,7 @@ struct PixelState {
 // scene at 1256x832, of a 4x4 block's half.)
 constexpr int kWarps = kRasterThreads / 32;
 constexpr int kGroup = 4;  // records blended at a time; a list is padded to it
-constexpr int kListLen = kChunk + kGroup;
+constexpr int kListLen = kChunk + 2 * kGroup;  // (and read a group ahead)
 // Dynamic shared memory: two staging buffers, a record that no pixel accepts
 // (the lists' padding), the records' block masks, and the half warps' lists.
 constexpr int kMaskOff = 2 * kBufBytes + kRecBytes;
@@ -398,9 +404,12 @@ __device__ __forceinline__ void blend_list(const unsigned char *__restrict__ aos
     }
     const uint32_t base = smem_addr(aos);
     uint32_t last = 0xffffu;  // offset of the last blended record
+    const uint32_t at = smem_addr(list);
+    static_assert(kGroup == 4, "a group's offsets are one 8-byte load");
+    uint2 next = lds_offsets(at);
     for (uint32_t m = 0; m < n; m += kGroup) {
-        static_assert(kGroup == 4, "a group's offsets are one 8-byte load");
-        const uint2 ii = *reinterpret_cast<const uint2 *>(list + m);
+        const uint2 ii = next;
+        next = lds_offsets(at + 2u * (m + kGroup));  // of the next group
         const uint32_t o[kGroup] = {ii.x & 0xffffu, ii.x >> 16, ii.y & 0xffffu, ii.y >> 16};
         float al[kGroup], w[kGroup], c[kGroup][3];
 #pragma unroll
