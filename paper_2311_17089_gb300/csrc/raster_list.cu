@@ -115,26 +115,14 @@ __device__ __forceinline__ uint32_t row_mask_of(const ListArgs &a, uint32_t g, i
     const float2 x = __ldg(reinterpret_cast<const float2 *>(a.rec + 3 * (size_t)g + 2) + 1);
     const uint32_t h0 = fabsf(u.x - cx0) <= x.x + kRowHalfX;
     const uint32_t h1 = fabsf(u.x - cx1) <= x.x + kRowHalfX;
-    const uint32_t halves = (h0 ? 0x55555555u : 0u) | (h1 ? 0xaaaaaaaau : 0u);
-    const float reach = x.y + kRowHalfY, y0 = (float)(ty * 16) + 0.5f;
-    auto hit = [&](int r) { return fabsf(u.y - (y0 + (float)r)) <= reach; };
-    if (!(fabsf(u.y) + reach < 1048576.0f)) {  // also NaN
-        uint32_t m = 0u;
-        for (int r = 0; r < 16; r++) m |= (hit(r) ? 3u : 0u) << (2 * r);
-        return m & halves;
+    uint32_t m = 0u;
+#pragma unroll
+    for (int r = 0; r < 16; r++) {
+        const float cy = (float)(ty * 16 + r) + 0.5f;
+        const uint32_t hit = fabsf(u.y - cy) <= x.y + kRowHalfY;
+        m |= (hit & h0) << (2 * r) | (hit & h1) << (2 * r + 1);
     }
-    // the rows hit are a run; below 2^20 its ends computed from the bounds
-    // are within one row, where the expression itself decides
-    const float lo = ceilf(u.y - reach - y0), hi = floorf(u.y + reach - y0);
-    int r0 = (int)fminf(fmaxf(lo, 0.0f), 16.0f), r1 = (int)fminf(fmaxf(hi, -1.0f), 15.0f);
-    if (r0 > 0 && hit(r0 - 1)) r0--;
-    else if (r0 < 16 && !hit(r0)) r0++;
-    if (r1 < 15 && hit(r1 + 1)) r1++;
-    else if (r1 >= 0 && !hit(r1)) r1--;
-    if (r0 > r1) return 0u;
-    // bits 2 r0 .. 2 r1 + 1
-    const uint32_t rows = (0xffffffffu << (2 * r0)) & (0xffffffffu >> (30 - 2 * r1));
-    return rows & halves;
+    return m;
 }
 
 // The half-row masks of the first kMaskPrefix entries of every tile list,
@@ -147,36 +135,19 @@ __global__ void __launch_bounds__(256) row_mask_kernel(ListArgs a) {
     const uint32_t c = blockIdx.x;
     if (a.use_list && *a.use_list == 0u) return;
     if (c >= a.seg_off[a.tiles]) return;
-    uint32_t lo = 0, hi = (uint32_t)a.tiles;  // seg_off[lo] <= c < seg_off[hi]
-    const uint32_t lane = threadIdx.x & 31u;
-    while (hi - lo > 1u) {  // a warp's lanes search together
-        const uint32_t step = (hi - lo + 31u) / 32u, q = lo + (lane + 1u) * step;
-        const uint32_t n = __popc(__ballot_sync(kFull, q < hi && __ldg(a.seg_off + q) <= c));
-        lo += n * step;
-        hi = min(hi, lo + step);
+    int lo = 0, hi = a.tiles;  // seg_off[lo] <= c < seg_off[hi]
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (a.seg_off[mid] <= c) lo = mid;
+        else hi = mid;
     }
-    const int t = (int)lo;
+    const int t = lo;
     const uint32_t L = a.seg_len[0];
     const uint32_t beg = a.ranges[2 * t], end = a.ranges[2 * t + 1];
     const uint32_t s0 = beg + (c - a.seg_off[t]) * L;
     const uint32_t s1 = min(min(end, s0 + L), beg + kMaskPrefix);
-    // bound by the latency of the dependent loads (index, then record):
-    // kMaskAhead entries of a thread are in flight (with the joint search
-    // and the masks' rows as runs, a 157x104 frame of 1M Gaussians 196 ->
-    // 193 us, 32 served requests 7.11 -> 6.99 ms)
-    constexpr int kMaskAhead = 4;
-    for (uint32_t e0 = s0 + threadIdx.x; e0 < s1; e0 += 256u * kMaskAhead) {
-        uint32_t g[kMaskAhead], m[kMaskAhead];
-#pragma unroll
-        for (int k = 0; k < kMaskAhead; k++)
-            g[k] = e0 + 256u * k < s1 ? __ldg(a.gidx + e0 + 256u * k) : 0u;
-#pragma unroll
-        for (int k = 0; k < kMaskAhead; k++)
-            m[k] = e0 + 256u * k < s1 ? row_mask_of(a, g[k], t) : 0u;
-#pragma unroll
-        for (int k = 0; k < kMaskAhead; k++)
-            if (e0 + 256u * k < s1) a.rowmask[e0 + 256u * k] = m[k];
-    }
+    for (uint32_t e = s0 + threadIdx.x; e < s1; e += 256u)
+        a.rowmask[e] = row_mask_of(a, __ldg(a.gidx + e), t);
 }
 
 // One pixel's blend state, held by every lane of its warp: T and the
