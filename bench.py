@@ -41,24 +41,29 @@ FP32_LANES_PER_SM = 128    # nominal, for the derived peak shown beside the meas
 OPS_PER_EVAL = 16          # FP32 operations per pixel-Gaussian evaluation
 # FP32 operations per pixel-Gaussian evaluation of the raster backward (an
 # FMA counting as one): the forward's alpha again (power 6, test 2, ex2 and
-# clamp 3), the colour and transmittance recurrences (F 3, T 2, 1 / (1 -
-# alpha) 2), dL/dalpha over the three channels (13), the opacity and power
-# terms (4), the centre and conic terms (18) and the pixel's share of the
-# warp's reduce-scatter of the 2D gradients (6)
-OPS_PER_BWD_EVAL = 60
+# clamp 3), the colour against dL/dC (3), the weight and the recurrences of
+# the colour behind and of T (4), 1 / (1 - alpha) (2), dL/dalpha and
+# dL/dpower (3), and the pixel's share of the record's nine sums (7)
+OPS_PER_BWD_EVAL = 30
 MUFU_LANES_PER_SM = 16     # nominal ex2 results per SM per clock (one ex2 per evaluation)
 PAPER_LEVEL_MIX = (0.95, 0.035, 0.01, 0.005)   # coarse levels under 5% of the Gaussians
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of ncu captures,
 # each with the SHA-256 (first 16 hex digits) of the kernel sources it was
 # taken on: a figure whose sources changed since is reported as stale (null)
-# (the raster figure was taken on sources whose kernels are those of the
-# current ones: since then only comments and the host's launch choice for
-# duplicate capacities below 1024 per tile, which no profiled frame has,
-# changed)
 RASTER_DRAM = {"bytes": 33.95e6, "sources": ("raster.cu", "raster_list.cu", "raster_ws.cuh"),
                "sha16": "d0db282cefbd654c"}   # mean over the 8 frames' raster stages, each frame alone
 PROJECT_VIEWS_DRAM = {"bytes": 505.1e6, "sources": ("project.cu", "footprint.cuh"),
                       "sha16": "1e94d3f932b66c6a"}   # the selective sweep's projection launch
+
+
+def bin_launches(n, tiles, cap, sms, own_sort):
+    """Kernels ms_bin (own_sort) or ms_bin_ordered launches: the start kernel,
+    the depth sort (one launch up to 4096 Gaussians, else 4 passes), the
+    items, the counts (which also sum the columns of a small matrix), the
+    columns, the ranks."""
+    rows = min(4 * sms, -(-cap // 2048))
+    fused = tiles <= 1024 and rows * tiles <= 16384
+    return 1 + ((1 if n <= 4096 else 4) if own_sort else 0) + 3 + (0 if fused else 1)
 
 
 def sources_sha16(names) -> str:
@@ -394,7 +399,7 @@ def train_step_bench(msgs, torch, ds, sc, dev, steps, warmup):
         # and list kernel; tile kernel; or, in between, both and the mask pass)
         blend = (2 if tiles < sms_dev else
                  3 if tiles < 4 * sms_dev and r.dup_capacity >= 1024 * tiles else 1)
-        launches += (1 + 4 + 1 + (1 if tiles <= 256 else 2) + 1) + 1 + blend + 1
+        launches += bin_launches(sc.n, tiles, r.dup_capacity, sms_dev, True) + 1 + blend + 1
     launches += 2                                   # batched backward: raster, projection
     nv = len(cams)
     # the projection pass: per Gaussian its geometry (44 B), the 2D gradients
@@ -1296,8 +1301,8 @@ def main():
         st_ = stats[("selective", cam.width)]
         bin_bytes += 44 * st_["survivors"] + 44 * st_["D"]
     roof_bin = {"bound": "hbm", "kernel": "the step's binning on one stream (the shared depth "
-                                          "sort and split, per frame start, duplicate, 1-2 tile "
-                                          "passes, ranges)",
+                                          "sort and split, per frame start, items, counts, "
+                                          "columns, ranks)",
                 "achieved": bin_bytes / (stage_ms["bin"] / 1e3) / 1e9, "peak": hbm_peak,
                 "unit": "GB/s", "bytes_per_step": bin_bytes}
     roof_bin["frac"] = roof_bin["achieved"] / hbm_peak
@@ -1397,9 +1402,8 @@ def main():
                            "images read back per frame"}
 
     # kernels of libmsgs per selective step: one projection for every frame,
-    # 4 passes of the shared depth sort and its split; per frame the start
-    # kernel, 4 depth passes (frames outside the shared order), duplicate,
-    # 1-2 tile passes, ranges; segment offsets, then the blend as ms_raster
+    # 4 passes of the shared depth sort and its split; per frame the binning
+    # (bin_launches); segment offsets, then the blend as ms_raster
     # launches it: the mask pass and the list kernel (fewer tiles than SMs),
     # the tile kernel alone (capped, or 4x as many tiles, or a capacity below
     # 1024 per tile), or both kernels and the mask pass (in between)
@@ -1410,8 +1414,8 @@ def main():
         cap_ok = rs_mode["selective"][k].dup_capacity >= 1024 * tiles
         blend = (2 if tiles < sms_dev else
                  3 if (not capped and tiles < 4 * sms_dev and cap_ok) else 1)
-        launches_per_step += (1 + (0 if k in sel_views else 4) + 1
-                              + (1 if tiles <= 256 else 2) + 1) + 1 + blend
+        launches_per_step += bin_launches(sc.n, tiles, rs_mode["selective"][k].dup_capacity,
+                                          sms_dev, k not in sel_views) + 1 + blend
 
     serve = None
     if not args.no_serve:

@@ -296,7 +296,7 @@ size_t ms_bin_workspace_bytes(int64_t n, int64_t tiles, int64_t dup_capacity);
  * listed for it in the order of their view depth).  n <= 2^30 - 1 (the
  * radix passes' digit counts are 30-bit).  Listed Gaussians are sorted by depth
  * bits with a stable LSD radix sort (ties keep index order), expanded to
- * one entry per covered tile in that order, and stably radix-sorted by tile
+ * one entry per covered tile in that order, and stably sorted by tile
  * id, which yields every tile's list in (depth, index) order.  Fully
  * asynchronous; D is only known on the device: entries beyond
  * dup_capacity are dropped and status bit 1 set.  `ws` (16-B aligned) of
@@ -705,9 +705,9 @@ int ms_serve_destroy(ms_server_t *srv);
 
 /*
  * Test hook for the bounded device waits (the paper has no counterpart):
- * every look-back wait of ms_bin (the radix passes' and the duplication's
- * decoupled look-back) gives up after `limit` polls of a predecessor that
- * has not published, instead of the default (about half a second), sets
+ * every look-back wait of ms_bin (the radix passes' decoupled look-back; up
+ * to 4096 Gaussians are sorted without one) gives up after `limit` polls of
+ * a predecessor that has not published, instead of the default (about half a second), sets
  * status bit 2 in ms_bins_t.counts and carries on with in-bounds writes;
  * ms_bin_counts then returns MS_ERR_TIMEOUT and the lists are not valid.
  * limit = 0 restores the default.  Process-wide; read when ms_bin enqueues
