@@ -19,6 +19,13 @@
 // and the weight of its 64 pixels for 16 records in shared memory and then
 // sums them with a record per lane (two lanes a record); the CTA adds each
 // record's sums to the per-Gaussian 2D gradient with one atomic per value.
+// The colour behind is the difference of the final colour and the colour
+// accumulated through the record, both rounded as the forward rounds them,
+// per channel.  As one running product with dL/dC (a tenth fewer
+// instructions) each step's rounding would stay in it while it shrinks to
+// nothing: the gradient of a record behind which nothing is left was up to
+// 2e-6 off instead of below 1e-6, and the 1M scene's opacities 1.7 times as
+// far from FP64.
 //
 // project_bwd_kernel: per Gaussian, the chain rule from (centre, conic,
 // opacity, colour) through V' = V + 0.3 I, V = J W Sigma W^T J^T, the
@@ -75,11 +82,10 @@ struct BwdArgs {
 };
 
 // A thread takes two pixels, (x, y) and (x, y + 4) of its warp's 8x8 block,
-// as packed FP32x2 pairs: T, the colour still behind weighted by dL/dC, R =
-// sum_c dL/dC_c (C_c - F_c), and dL/dC.  With g = sum_c dL/dC_c c_k,c of
-// record k, R_k = R_{k-1} - w_k g and dL/dalpha_k = T_k g - R_k / (1 - alpha_k).
+// as packed FP32x2 pairs: T, the colour F accumulated so far, the final
+// colour C and dL/dC.
 struct PixPair {
-    f32x2 T, R, d0, d1, d2;
+    f32x2 T, F0, F1, F2, C0, C1, C2, d0, d1, d2;
     int cntA, cntB;  // entries of the segment each pixel blended through
 };
 
@@ -129,58 +135,65 @@ __device__ __forceinline__ bool reaches_block(const float4 r0, float C, const fl
 
 // The nine sums of the warp's first n slots, a record per lane pair (lane
 // and lane + 16 take 32 pixels each): the pixels' weights against dL/dC, and
-// the moments of dL/dpower about the block's centre (bcx, bcy), shifted to
-// the record's.  Added to the CTA's sums.
+// the moments of dL/dpower about the record's centre.  Added to the CTA's
+// sums.  (bcx, bcy): the block's centre.  About the record's own centre: the
+// second moments of a splat smaller than a pixel, taken about the block's
+// centre and shifted, are differences of terms a hundred times their size.
 __device__ __forceinline__ void add_slots(const BwdWarp &wp, uint32_t n, const float4 *rec,
                                           float bcx, float bcy, float (*acc)[kG2 + 1]) {
     const uint32_t lane = threadIdx.x & 31u, r = lane & 15u, h = lane >> 4;
     const float *q = wp.q + h * kHalfF + r, *w = wp.w + h * kHalfF + r;
     const float4 *d = wp.d + 32 * h;
+    // lanes without a record sum slots that nothing reads; their centre is
+    // any staged record's
+    const uint32_t j = r < n ? wp.slot[r] : wp.slot[0];
+    const float4 r0 = rec[3 * j];
+    const float2 r1 = *reinterpret_cast<const float2 *>(rec + 3 * j + 1);
+    float X[8], XX[8];  // pixel columns from the record's centre
+#pragma unroll
+    for (int x = 0; x < 8; x++) {
+        X[x] = (bcx + ((float)x - 3.5f)) - r0.x;
+        XX[x] = X[x] * X[x];
+    }
     float m0 = 0.0f, mx = 0.0f, my = 0.0f, mxx = 0.0f, mxy = 0.0f, myy = 0.0f;
     float w0 = 0.0f, w1 = 0.0f, w2 = 0.0f;
-    const float y0 = h ? 0.5f : -3.5f;
+    const float y0 = bcy + (h ? 0.5f : -3.5f);
 #pragma unroll
     for (int row = 0; row < 4; row++) {
-        float r0 = 0.0f, r1 = 0.0f, r2 = 0.0f;
+        float s0 = 0.0f, s1 = 0.0f, s2 = 0.0f;
 #pragma unroll
         for (int x = 0; x < 8; x++) {
             const int p = row * 8 + x;
-            const float X = (float)x - 3.5f;
             const float qv = q[p * kRowF], wv = w[p * kRowF];
             const float4 dv = d[p];
-            r0 += qv;
-            r1 = fmaf(qv, X, r1);
-            r2 = fmaf(qv, X * X, r2);
+            s0 += qv;
+            s1 = fmaf(qv, X[x], s1);
+            s2 = fmaf(qv, XX[x], s2);
             w0 = fmaf(wv, dv.x, w0);
             w1 = fmaf(wv, dv.y, w1);
             w2 = fmaf(wv, dv.z, w2);
         }
-        const float Y = y0 + (float)row;
-        m0 += r0;
-        mx += r1;
-        mxx += r2;
-        my = fmaf(Y, r0, my);
-        mxy = fmaf(Y, r1, mxy);
-        myy = fmaf(Y * Y, r0, myy);
+        const float Y = (y0 + (float)row) - r0.y;
+        m0 += s0;
+        mx += s1;
+        mxx += s2;
+        my = fmaf(Y, s0, my);
+        mxy = fmaf(Y, s1, mxy);
+        myy = fmaf(Y * Y, s0, myy);
     }
     float v[kG2] = {m0, mx, my, mxx, mxy, myy, w0, w1, w2};
 #pragma unroll
     for (int k = 0; k < kG2; k++) v[k] += __shfl_xor_sync(0xffffffffu, v[k], 16);
     if (r >= n) return;
-    const uint32_t j = wp.slot[r];
-    const float4 r0 = rec[3 * j];
-    const float2 r1 = *reinterpret_cast<const float2 *>(rec + 3 * j + 1);
-    const float dx = bcx - r0.x, dy = bcy - r0.y;
-    const float Dx = fmaf(dx, v[0], v[1]), Dy = fmaf(dy, v[0], v[2]);
     const float ca = r0.z * kInvConicA, cb = r0.w * kInvConicB, cc = r1.x * kInvConicA;
     // the first lane of a pair adds the centre and conic sums, the second
     // the opacity and colours
     if (h == 0) {
-        atomicAdd(&acc[j][0], ca * Dx + cb * Dy);
-        atomicAdd(&acc[j][1], cb * Dx + cc * Dy);
-        atomicAdd(&acc[j][2], -0.5f * fmaf(dx, Dx + v[1], v[3]));
-        atomicAdd(&acc[j][3], -(v[4] + dx * v[2] + dy * Dx));
-        atomicAdd(&acc[j][4], -0.5f * fmaf(dy, Dy + v[2], v[5]));
+        atomicAdd(&acc[j][0], ca * v[1] + cb * v[2]);
+        atomicAdd(&acc[j][1], cb * v[1] + cc * v[2]);
+        atomicAdd(&acc[j][2], -0.5f * v[3]);
+        atomicAdd(&acc[j][3], -v[4]);
+        atomicAdd(&acc[j][4], -0.5f * v[5]);
         acc[j][kG2] = 1.0f;
     } else {
         atomicAdd(&acc[j][5], v[0] / r1.y);
@@ -190,14 +203,15 @@ __device__ __forceinline__ void add_slots(const BwdWarp &wp, uint32_t n, const f
     }
 }
 
-// Bound by instruction issue.  A record costs a warp about 55 instructions
+// Bound by instruction issue.  A record costs a warp about 65 instructions
 // for its 64 pixels' gradients and 24 for the nine sums over them: those are
 // 9 x 64 products with per-pixel factors, formed 16 records at a time with a
 // record per lane, instead of nine reductions across the warp per record
-// (12 shuffles and about 70 instructions).  With the per-pixel state cut from
-// three colours to their product with dL/dC, records culled by their level
-// set instead of its box, and cp.async staging: the 4-view batch of 1M
-// Gaussians (1256x832, 314x208, 78x52, 19x13) 825 -> 606 us.
+// (12 shuffles and about 70 instructions).  With records culled by their
+// level set instead of its box, and cp.async staging: the 4-view batch of 1M
+// Gaussians (1256x832, 314x208, 78x52, 19x13) 820 -> 650 us; 590 with the
+// colour behind kept as one product and the moments about the block's
+// centre, which lost precision (add_slots and the head of this file).
 __global__ void __launch_bounds__(kBwdThreads, 4)
 raster_bwd_kernel(const __grid_constant__ BwdArgs args) {
     pdl_wait();
@@ -258,38 +272,47 @@ raster_bwd_kernel(const __grid_constant__ BwdArgs args) {
         const int tx = t % a.tiles_x, ty = t / a.tiles_x;
         const int px = tx * 16 + lx;
         PixPair pp;
-        float st[2][5];  // per pixel: T, R, d0..2
+        float st[2][10];  // per pixel: T, F0..2, C0..2, d0..2
         uint32_t cnt[2] = {0u, 0u};
 #pragma unroll
         for (int h = 0; h < 2; h++) {
             const int py = ty * 16 + (h ? lyB : lyA);
             st[h][0] = 1.0f;
 #pragma unroll
-            for (int q = 1; q < 5; q++) st[h][q] = 0.0f;
+            for (int q = 1; q < 10; q++) st[h][q] = 0.0f;
             if (px < a.W && py < a.H && len > 0) {
                 const size_t p = (size_t)py * a.W + px, plane = (size_t)a.W * a.H;
                 const uint32_t nc = a.n_contrib[p];
                 if (nc > pos0) {
                     cnt[h] = min(nc - pos0, len);
-                    float4 s4 = make_float4(0.0f, 0.0f, 0.0f, 1.0f);
-                    if (k > 0)
-                        s4 = __ldcg(a.pre + (size_t)(c - 1) * kRasterThreads + (h ? fB : fA));
-                    const float d0 = a.dl[p], d1 = a.dl[plane + p], d2 = a.dl[2 * plane + p];
-                    st[h][0] = s4.w;
-                    st[h][1] = d0 * (a.image[p] - s4.x) + d1 * (a.image[plane + p] - s4.y) +
-                               d2 * (a.image[2 * plane + p] - s4.z);
-                    st[h][2] = d0;
-                    st[h][3] = d1;
-                    st[h][4] = d2;
+                    if (k > 0) {
+                        const float4 s4 =
+                            __ldcg(a.pre + (size_t)(c - 1) * kRasterThreads + (h ? fB : fA));
+                        st[h][0] = s4.w;
+                        st[h][1] = s4.x;
+                        st[h][2] = s4.y;
+                        st[h][3] = s4.z;
+                    }
+                    st[h][4] = a.image[p];
+                    st[h][5] = a.image[plane + p];
+                    st[h][6] = a.image[2 * plane + p];
+                    st[h][7] = a.dl[p];
+                    st[h][8] = a.dl[plane + p];
+                    st[h][9] = a.dl[2 * plane + p];
                 }
             }
-            wp.d[lane + 32 * h] = make_float4(st[h][2], st[h][3], st[h][4], 0.0f);
+            wp.d[lane + 32 * h] = make_float4(st[h][7], st[h][8], st[h][9], 0.0f);
         }
         pp.T = pack2(st[0][0], st[1][0]);
-        pp.R = pack2(st[0][1], st[1][1]);
-        pp.d0 = pack2(st[0][2], st[1][2]);
-        pp.d1 = pack2(st[0][3], st[1][3]);
-        pp.d2 = pack2(st[0][4], st[1][4]);
+        pp.F0 = pack2(st[0][1], st[1][1]);
+        pp.F1 = pack2(st[0][2], st[1][2]);
+        pp.F2 = pack2(st[0][3], st[1][3]);
+        pp.C0 = pack2(st[0][4], st[1][4]);
+        pp.C1 = pack2(st[0][5], st[1][5]);
+        pp.C2 = pack2(st[0][6], st[1][6]);
+        pp.d0 = pack2(st[0][7], st[1][7]);
+        pp.d1 = pack2(st[0][8], st[1][8]);
+        pp.d2 = pack2(st[0][9], st[1][9]);
         pp.cntA = (int)cnt[0];
         pp.cntB = (int)cnt[1];
         const float fx = (float)px + 0.5f;
@@ -352,21 +375,27 @@ raster_bwd_kernel(const __grid_constant__ BwdArgs args) {
                 const bool accB = (int)j < limB && pB <= 0.0f && pB >= r2.y;
                 if (!__any_sync(0xffffffffu, accA || accB)) continue;
                 // alpha of accepted pixels, 0 for the others (no effect on T,
-                // R or any gradient); gradients through alpha only below the
+                // F or any gradient); gradients through alpha only below the
                 // 0.99 clamp
                 const float GA = r1.y * ex2_approx_b(accA ? pA : -256.0f);
                 const float GB = r1.y * ex2_approx_b(accB ? pB : -256.0f);
                 const float alA = accA ? fminf(0.99f, GA) : 0.0f;
                 const float alB = accB ? fminf(0.99f, GB) : 0.0f;
-                const f32x2 al = pack2(alA, alB), nal = pack2(-alA, -alB);
+                const f32x2 al = pack2(alA, alB);
                 const f32x2 ag = pack2(GA < 0.99f ? alA : 0.0f, GB < 0.99f ? alB : 0.0f);
-                const f32x2 g = fma2(splat2(r2.x), pp.d2,
-                                     fma2(splat2(r1.w), pp.d1, mul2(splat2(r1.z), pp.d0)));
                 const f32x2 w = mul2(al, pp.T);
-                pp.R = fma2(mul2(nal, pp.T), g, pp.R);
+                const f32x2 c0 = splat2(r1.z), c1 = splat2(r1.w), c2 = splat2(r2.x);
+                pp.F0 = fma2(w, c0, pp.F0);
+                pp.F1 = fma2(w, c1, pp.F1);
+                pp.F2 = fma2(w, c2, pp.F2);
+                const f32x2 om = sub2(splat2(1.0f), al);
                 const f32x2 nio = pack2(-__fdividef(1.0f, 1.0f - alA), -__fdividef(1.0f, 1.0f - alB));
-                const f32x2 dal = fma2(pp.R, nio, mul2(pp.T, g));
-                pp.T = fma2(nal, pp.T, pp.T);
+                // dC/dalpha = T c - (C - F) / (1 - alpha), summed over channels with dL/dC
+                const f32x2 t0 = fma2(sub2(pp.C0, pp.F0), nio, mul2(pp.T, c0));
+                const f32x2 t1 = fma2(sub2(pp.C1, pp.F1), nio, mul2(pp.T, c1));
+                const f32x2 t2 = fma2(sub2(pp.C2, pp.F2), nio, mul2(pp.T, c2));
+                const f32x2 dal = fma2(pp.d2, t2, fma2(pp.d1, t1, mul2(pp.d0, t0)));
+                pp.T = mul2(pp.T, om);
                 float q0, q1, w0, w1;
                 unpack2(mul2(dal, ag), q0, q1);  // dL/dpower
                 unpack2(w, w0, w1);
