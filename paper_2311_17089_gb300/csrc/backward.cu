@@ -742,17 +742,6 @@ project_bwd_kernel(const __grid_constant__ ProjBwdArgs p) {
     for (int64_t i0 = ((int64_t)blockIdx.x * kProjBwdWarps + wid) * 32; i0 < n; i0 += warps * 32) {
         const int64_t i = i0 + lane;
         const int rows = (int)min((int64_t)32, n - i0);
-        const float *gcol = p.sc.color + i0 * CR::RS;
-        float *gdc = p.out.dcolor + i0 * CR::RS;
-        // the colour rows, copied while the 2D gradients are read: both loads
-        // were waited for in turn (4 views of 1M Gaussians, whole training
-        // step: 2019 -> 2008 us, 1967 -> 1956 us)
-        for (int e = lane; e < rows * CR::RS; e += 32) {
-            const int r = e / CR::RS, col = e - r * CR::RS;
-            cp_async4(s_coef + r * CR::STRIDE + col, gcol + e);
-            if (acc) cp_async4(s_dcol + r * CR::STRIDE + col, gdc + e);
-            else s_dcol[r * CR::STRIDE + col] = 0.0f;
-        }
         uint32_t vmask = 0;  // views that blended this lane's Gaussian
         if (i < n) {
             for (int k = 0; k < p.n_views; k++) {
@@ -764,10 +753,17 @@ project_bwd_kernel(const __grid_constant__ ProjBwdArgs p) {
             }
         }
         const bool warp_any = __any_sync(0xffffffffu, vmask != 0);
-        cp_async_commit();
-        cp_async_wait<0>();
-        __syncwarp();
         if (!warp_any && acc) continue;
+        const float *gcol = p.sc.color + i0 * CR::RS;
+        float *gdc = p.out.dcolor + i0 * CR::RS;
+        if (warp_any) {
+            for (int e = lane; e < rows * CR::RS; e += 32) {
+                const int r = e / CR::RS, col = e - r * CR::RS;
+                s_coef[r * CR::STRIDE + col] = gcol[e];
+                s_dcol[r * CR::STRIDE + col] = acc ? gdc[e] : 0.0f;
+            }
+        }
+        __syncwarp();
         float dm[3] = {0.0f, 0.0f, 0.0f}, dls[3] = {0.0f, 0.0f, 0.0f};
         float dq[4] = {0.0f, 0.0f, 0.0f, 0.0f}, dop = 0.0f;
         // each lane walks its own views in ascending order (the order of the

@@ -50,10 +50,6 @@ __device__ __forceinline__ void cp_async16(void *dst, const void *src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(dst)), "l"(src)
                  : "memory");
 }
-__device__ __forceinline__ void cp_async4(void *dst, const void *src) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_addr(dst)), "l"(src)
-                 : "memory");
-}
 // Arrives on the mbarrier (one of its initial count) once the thread's
 // cp_async16 copies so far have landed.
 __device__ __forceinline__ void cp_async_arrive(uint64_t *bar) {
