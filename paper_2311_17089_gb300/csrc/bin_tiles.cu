@@ -92,8 +92,7 @@ struct ItemsK {
     const uint32_t *order, *n32, *n_tiles;
     const uint2 *rect;
     uint32_t n_max;
-    int tiles_x;
-    uint32_t tiles;
+    uint32_t tiles_x, tiles;
     uint32_t block_size;
     bool vec;  // the order is 16-byte aligned
     Blocks b;
@@ -145,7 +144,14 @@ __global__ void __launch_bounds__(kItemThreads) tile_items_kernel(ItemsK a) {
         uint32_t se = 0, sc = 0;
 #pragma unroll
         for (int r = 0; r < kItemIPT; r++) {
-            if (nt[r] > a.tiles) nt[r] = 0u;  // not a count ms_project wrote for this frame
+            // not a count or a first tile that ms_project wrote for this frame
+            // (it writes them for its own camera's): reported, and left out
+            if (nt[r] > a.tiles ||
+                (nt[r] && (rc[r].x >> 16) * a.tiles_x + (rc[r].x & 0xffffu) >= a.tiles)) {
+                MS_DCHECK(false, a.err);
+                atomicOr(a.err, (unsigned long long)kStatusTimeout);
+                nt[r] = 0u;
+            }
             se += nt[r];
             sc += nt[r] != 0u;
         }
@@ -172,7 +178,7 @@ __global__ void __launch_bounds__(kItemThreads) tile_items_kernel(ItemsK a) {
             const uint32_t x0 = rc[r].x & 0xffffu, y0 = rc[r].x >> 16;
             const uint32_t w1 = (rc[r].y & 0xffffu) - x0;
             a.item[p] = make_uint2((uint32_t)min(e, (unsigned long long)kClip),
-                                   ((y0 * (uint32_t)a.tiles_x + x0) & 0xffffu) | (w1 << 16));
+                                   (y0 * a.tiles_x + x0) | (w1 << 16));
             a.idx[p] = g[r];
             p++;
             e += nt[r];
@@ -783,7 +789,7 @@ int launch_tile_lists(const TileListArgs &t, cudaStream_t st) {
     ik.n_tiles = t.n_tiles;
     ik.rect = t.rect;
     ik.n_max = (uint32_t)t.n;
-    ik.tiles_x = t.tiles_x;
+    ik.tiles_x = (uint32_t)t.tiles_x;
     ik.tiles = (uint32_t)t.tiles;
     ik.block_size = (uint32_t)size;
     ik.vec = aligned(t.order, 16);
