@@ -42,6 +42,7 @@
 #include "common.cuh"
 #include "f32x2.cuh"
 #include "raster_ws.cuh"
+#include "reach.cuh"
 #include "tma.cuh"
 
 namespace msgs {
@@ -110,17 +111,17 @@ struct BwdSmem {
 };
 
 // The record's alpha can reach 1/255 at some pixel centre of the 8x8 block
-// centred on (cx, cy): its level-set box reaches the block, and so does the
-// level set itself (power log2(e) = A dx^2 + B dx dy + C dy^2 is concave, so
-// over a rectangle that does not hold the centre its maximum lies on the
-// side nearest in x or the one nearest in y, at a clamped division).  The
+// centred on (cx, cy): power log2(e) = A dx^2 + B dx dy + C dy^2 is concave,
+// so over a rectangle that does not hold the centre its maximum lies on the
+// side nearest in x or the one nearest in y, at a clamped division.  The
 // margin covers the rounding of this evaluation and of the pixels', each a
-// few 2^-24 of the terms' magnitudes; NaN keeps the record.
-__device__ __forceinline__ bool reaches_block(const float4 r0, float C, const float4 r2, float cx,
+// few 2^-24 of the terms' magnitudes.  A conic that is not concave beyond the
+// rounding (reach.cuh), and NaN, keep the record.
+__device__ __forceinline__ bool reaches_block(const float4 r0, float C, float thr, float cx,
                                               float cy) {
-    constexpr float kHalf = 3.5f, kReach = 3.5625f;
-    if (!(fabsf(r0.x - cx) <= r2.z + kReach && fabsf(r0.y - cy) <= r2.w + kReach)) return false;
+    constexpr float kHalf = 3.5f;
     const float A = r0.z, B = r0.w;
+    if (!(reach_curved(A, C) && reach_det(A, B, C) > 0.0f)) return true;
     const float xl = cx - kHalf - r0.x, xh = cx + kHalf - r0.x;
     const float yl = cy - kHalf - r0.y, yh = cy + kHalf - r0.y;
     const float xn = fmaxf(xl, fminf(0.0f, xh)), yn = fmaxf(yl, fminf(0.0f, yh));
@@ -130,7 +131,7 @@ __device__ __forceinline__ bool reaches_block(const float4 r0, float C, const fl
     const float p2 = (A * xs + B * yn) * xs + C * yn * yn;
     const float X = fmaxf(fabsf(xl), fabsf(xh)), Y = fmaxf(fabsf(yl), fabsf(yh));
     const float m = 1.52587890625e-5f * (fabsf(A) * X * X + fabsf(B) * X * Y + fabsf(C) * Y * Y);
-    return !(fmaxf(p1, p2) < r2.y - m);
+    return !(fmaxf(p1, p2) < thr - m);
 }
 
 // The nine sums of the warp's first n slots, a record per lane pair (lane
@@ -352,7 +353,7 @@ raster_bwd_kernel(const __grid_constant__ BwdArgs args) {
             for (uint32_t j0 = 0; j0 < jn; j0 += 32) {
                 const uint32_t j = j0 + lane;
                 const bool rel = j < jn && reaches_block(rec[3 * j], rec[3 * j + 1].x,
-                                                         rec[3 * j + 2], bcx, bcy);
+                                                         rec[3 * j + 2].y, bcx, bcy);
                 const uint32_t m = __ballot_sync(0xffffffffu, rel);
                 if (rel) wp.list[nl + __popc(m & ((1u << lane) - 1u))] = (uint16_t)j;
                 nl += __popc(m);

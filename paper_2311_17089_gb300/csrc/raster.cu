@@ -50,6 +50,7 @@
 #include "tma.cuh"
 #include "raster_ws.cuh"
 #include "raster_list.cuh"
+#include "reach.cuh"
 
 namespace msgs {
 
@@ -78,12 +79,6 @@ constexpr uint32_t kListMeanMax = 8192;
 __device__ __forceinline__ float ex2_approx(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-
-__device__ __forceinline__ float sqrt_approx(float x) {
-    float y;
-    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
 
@@ -268,9 +263,9 @@ constexpr int kListLen = kChunk + 2 * kGroup;  // (and read a group ahead)
 constexpr int kMaskOff = 2 * kBufBytes + kRecBytes;
 constexpr int kListOff = kMaskOff + kChunk * 2;
 constexpr int kSmemBytes = kListOff + kWarps * 2 * kListLen * 2;
-// A record's half extents bound the exact alpha >= 1/255 level set; the
-// rounding of that bound, of the chords below and of the distances is below
-// 1e-3 px at the largest image coordinates.
+// The chords and extents below bound the pixels a record is accepted at
+// (reach.cuh); the margin covers the rounding of their own last operations
+// and of the distances (a few 2^-24 of the record's extents: 0.06 px at 10^5).
 #ifndef MS_CULL_MARGIN
 #define MS_CULL_MARGIN 0.0625f
 #endif
@@ -278,34 +273,38 @@ constexpr float kInf = __builtin_huge_valf();
 
 // Bits 4 k + j, k = 0, 1: some pixel centre of the tile's 4x4 block (j, row
 // band b0 + k) may have alpha >= 1/255.  (x, y): the record's centre relative
-// to the tile's corner.  Over a band of pixel rows the level set {A dx^2 +
-// B dx dy + C dy^2 >= thr} spans an x interval whose ends are chords' ends:
-// the right end is largest at the row of the set's rightmost point (dx = ex,
-// dy = -B ex / 2C), so over the band at the nearest row to that; the left
-// end likewise with the signs turned.  The discriminant is raised by more
-// than its rounding; a conic without usable curvature, or NaN, keeps every
-// block that the box reaches.
+// to the tile's corner.  Over a band of pixel rows the rows' intervals of
+// reach.cuh span an x interval whose ends are chords' ends: the right end
+// is largest at the row of the ellipse's rightmost point (dx = ex, dy = -B ex /
+// 2C), so over the band at the nearest row to that; the left end likewise
+// with the signs turned.  Without an ellipse a chord's end is a convex
+// function of its row, largest at the band's first or last.  A conic without
+// usable curvature, or NaN, keeps every block.
 __device__ __forceinline__ uint32_t blocks_reached(float x, float y, float A, float B, float C,
-                                                   float thr, float ex, float ey, int b0) {
+                                                   float thr, int b0) {
+    if (!reach_curved(A, C)) return 0xffu;
+    float ex, ey;
+    const bool bounded = reach_extents(A, B, C, thr, ex, ey);
+    const float den = reach_det(A, B, C), top = A * reach_thr(thr);
     const float yr = -0.5f * ex * __fdividef(B, C);  // dy of the rightmost point
-    const float ia = __fdividef(-0.5f, A);
-    const bool flat = !(A < -1e-30f) || !(C < -1e-30f);
+    const float ia = __fdividef(-0.5f, A), slope = ia * B;
     uint32_t bits = 0u;
 #pragma unroll
     for (int k = 0; k < 2; k++) {
         // the band's pixel centres relative to the record's
         const float yl = (float)(4 * (b0 + k)) + 0.5f - y, yh = yl + 3.0f;
-        if (yl > ey + MS_CULL_MARGIN || yh < -ey - MS_CULL_MARGIN) continue;
-        float x1 = ex, x0 = -ex;
-        if (!flat) {
-            auto chord = [&](float dy, float sign) {  // the end of the chord at dy
-                const float h = B * dy, t = 4.0f * A * (C * dy * dy - thr);
-                const float d = h * h - t + 3.8e-6f * (h * h + fabsf(4.0f * A * C * dy * dy) + fabsf(4.0f * A * thr));
-                return ia * (h + sign * sqrt_approx(fmaxf(d, 0.0f)));
-            };
+        auto chord = [&](float dy, float side) {  // the end of the chord at dy
+            return fmaf(side, sqrt_approx(fmaxf(fmaf(-den, dy * dy, top), 0.0f)), slope * dy);
+        };
+        float x1, x0;
+        if (bounded) {
+            if (yl > ey + MS_CULL_MARGIN || yh < -ey - MS_CULL_MARGIN) continue;
             const float r = fminf(yh, fmaxf(yl, yr)), l = fminf(yh, fmaxf(yl, -yr));
-            if (r != yr) x1 = chord(r, 1.0f);
-            if (l != -yr) x0 = chord(l, -1.0f);
+            x1 = r != yr ? chord(r, ia) : ex;
+            x0 = l != -yr ? chord(l, -ia) : -ex;
+        } else {
+            x1 = fmaxf(chord(yl, ia), chord(yh, ia));
+            x0 = fminf(chord(yl, -ia), chord(yh, -ia));
         }
         x1 += x + MS_CULL_MARGIN;
         x0 += x - MS_CULL_MARGIN;
@@ -586,9 +585,10 @@ __device__ __forceinline__ int run_segment(const RasterArgs &a, const Seg &sg, u
             const uint32_t i = tid & (uint32_t)(kChunk - 1), band = (tid / kChunk) * 2u;
             uint32_t bits = 0u;
             if (i < cnt) {
-                const float4 r0 = buf[3 * i], r1 = buf[3 * i + 1], r2 = buf[3 * i + 2];
+                const float4 r0 = buf[3 * i], r1 = buf[3 * i + 1];
+                const float2 r2 = *reinterpret_cast<const float2 *>(buf + 3 * i + 2);
                 bits = blocks_reached(r0.x - (float)(tx * 16), r0.y - (float)(ty * 16), r0.z, r0.w,
-                                      r1.x, r2.y, r2.z, r2.w, (int)band);
+                                      r1.x, r2.y, (int)band);
                 // B^2 below 4 A C by more than the power's rounding, a few
                 // 2^-24 of its terms: it cannot come out positive
                 bad = !((r1.z + r1.w + r2.x) * 0.0f == 0.0f) ||

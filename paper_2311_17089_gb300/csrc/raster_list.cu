@@ -41,6 +41,7 @@
 #include "common.cuh"
 #include "raster_list.cuh"
 #include "raster_ws.cuh"
+#include "reach.cuh"
 #include "tma.cuh"
 
 namespace msgs {
@@ -59,11 +60,8 @@ constexpr int kStageF4 = 3 * kCullWin;
 constexpr int kPosOff = 2 * kStageF4 * 16;
 constexpr int kCntOff = kPosOff + 2 * kCullWin * 2;
 constexpr int kListSmem = kCntOff + kCullPerThread * kListPixelsPerCta * 4;
-// Half extents of the row's pixel centres (8 x 1) plus the margin the tile
-// kernel's per-warp culling uses for FP32 rounding: the record's half
-// extents bound the exact alpha >= 1/255 level set, and the rounding of
-// that bound and of the distances is below 1e-4 px at the largest image
-// coordinates.
+// Half extents of the row's pixel centres (8 x 1) plus a margin for the
+// rounding of the distances (reach.cuh bounds the accepted pixels).
 constexpr float kRowHalfX = 3.5f + 0.0625f;
 constexpr float kRowHalfY = 0.0625f;
 
@@ -101,18 +99,21 @@ __device__ __forceinline__ uint32_t window_end(uint32_t p, uint32_t L, uint32_t 
 // reaches beyond it has its mask formed by the blend's own thread.
 constexpr uint32_t kMaskPrefix = 16384;
 
-// Bit 2 r + h: the level-set box of the entry for Gaussian g, widened by
-// the half extents of a half row, reaches the centre of the pixels (16 tx +
-// 8 h + 0..7, 16 ty + r) of tile t = (tx, ty).  The FP32 expression is the
-// one the blend assumes, the same for every half row.
+// Bit 2 r + h: the box of the pixels that can accept the entry for Gaussian
+// g (reach_extents; without bounded extents every row), widened by the half
+// extents of a half row, reaches the centre of the pixels (16 tx + 8 h +
+// 0..7, 16 ty + r) of tile t = (tx, ty).  The FP32 expression is the one the
+// blend assumes, the same for every half row.
 __device__ __forceinline__ uint32_t row_mask_of(const ListArgs &a, uint32_t g, int t) {
     const int tx = t % a.tiles_x, ty = t / a.tiles_x;
     const float cx0 = (float)(tx * 16) + 4.0f, cx1 = (float)(tx * 16 + 8) + 4.0f;
     MS_DCHECK(g < a.n_rec, a.err);
     if (g >= a.n_rec) g = 0;  // unreachable unless binning reported an error
-    // the centre (r0.xy) and the half extents (r2.zw)
-    const float2 u = __ldg(reinterpret_cast<const float2 *>(a.rec + 3 * (size_t)g));
-    const float2 x = __ldg(reinterpret_cast<const float2 *>(a.rec + 3 * (size_t)g + 2) + 1);
+    // the centre, the conic and the threshold
+    const float4 u = __ldg(a.rec + 3 * (size_t)g);
+    const float C = __ldg(&a.rec[3 * (size_t)g + 1].x), thr = __ldg(&a.rec[3 * (size_t)g + 2].y);
+    float2 x;
+    if (!reach_extents(u.z, u.w, C, thr, x.x, x.y)) return 0xffffffffu;
     const uint32_t h0 = fabsf(u.x - cx0) <= x.x + kRowHalfX;
     const uint32_t h1 = fabsf(u.x - cx1) <= x.x + kRowHalfX;
     uint32_t m = 0u;
