@@ -116,7 +116,7 @@ onesweep_pass(PassArgs a) {
         for (int r = 0; r < IPT; r++) {
             const uint32_t i = wbase + (uint32_t)r * 32u + lane;
             ok[r] = i < n;
-            if (a.filter && ok[r]) ok[r] = __ldg(a.filter + i) > 0;
+            if (a.filter && ok[r]) ok[r] = a.filter[i] > 0;
         }
 #pragma unroll
         for (int r = 0; r < IPT; r++) {
@@ -379,10 +379,9 @@ block_sort_kernel(const uint32_t *__restrict__ keys, const uint32_t *__restrict_
 // projection's own status and (ms_bin_ordered) the status of the depth sort
 // it takes its order from.  Every later kernel of the call only ORs into
 // the status word, after this one.
-__global__ void bin_start_kernel(const uint32_t *__restrict__ stats,
-                                 const uint32_t *__restrict__ order_stats,
-                                 unsigned long long *__restrict__ counts, uint64_t cap,
-                                 uint4 *__restrict__ zero16, uint64_t n16) {
+__global__ void bin_start_kernel(const uint32_t *stats, const uint32_t *order_stats,
+                                 unsigned long long *counts, uint64_t cap, uint4 *zero16,
+                                 uint64_t n16) {
     pdl_wait();
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     const uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;

@@ -248,9 +248,9 @@ __device__ __forceinline__ void walk_items(const PartsK &a, const uint32_t *pre,
             v1 = make_uint2(kClip, 0u);
             n1 = total;
             if (q < kept) {
-                v1 = __ldg(item + q);
-                if (kIdx) g1 = __ldg(idx + q);
-                if (q + 1u < kept) n1 = __ldg(&item[q + 1u].x);
+                v1 = item[q];
+                if (kIdx) g1 = idx[q];
+                if (q + 1u < kept) n1 = item[q + 1u].x;
             }
         };
         load(i + lane);
@@ -298,7 +298,7 @@ __global__ void __launch_bounds__(32 * kWarps, kCtasPerSm) tile_count_kernel(Par
         const uint32_t b0 = min(n_blocks, tid * per), b1 = min(n_blocks, b0 + per);
         unsigned long long sum = 0;
 #pragma unroll 8
-        for (uint32_t b = b0; b < b1; b++) sum += __ldg(a.b.sum + b);
+        for (uint32_t b = b0; b < b1; b++) sum += a.b.sum[b];
         unsigned long long x = sum;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -311,7 +311,7 @@ __global__ void __launch_bounds__(32 * kWarps, kCtasPerSm) tile_count_kernel(Par
         for (uint32_t k = 0; k < w; k++) run += s_scan[k];
         for (uint32_t b = b0; b < b1; b++) {
             s_pre[b] = (uint32_t)min(run, (unsigned long long)kClip);
-            run += __ldg(a.b.sum + b);
+            run += a.b.sum[b];
         }
         if (tid == blockDim.x - 1u) s_pre[n_blocks] = (uint32_t)min(run, (unsigned long long)kClip);
         __syncthreads();
@@ -350,7 +350,7 @@ __global__ void __launch_bounds__(32 * kWarps, kCtasPerSm) tile_count_kernel(Par
             uint32_t l = 0, h = a.b.kept[b];  // item[l] starts before f0
             while (h - l > 1u) {
                 const uint32_t step = (h - l + 31u) / 32u, q = l + (lane + 1u) * step;
-                const uint32_t c = __popc(__ballot_sync(kAll, q < h && __ldg(&item[q].x) < f0));
+                const uint32_t c = __popc(__ballot_sync(kAll, q < h && item[q].x < f0));
                 l += c * step;
                 h = min(h, l + step);
             }

@@ -117,6 +117,12 @@ __device__ __forceinline__ void fence_acquire() {
 // visible.  It also lets the next kernel's launch begin.  Between the
 // dozen short dependent kernels of a frame this hides the launch and the
 // CTAs' start, 1-3 us each.
+// What the kernel before wrote is read by plain or .cg loads, never by
+// ld.global.nc (__ldg, or a const __restrict__ parameter), which wants data
+// that no one writes while the reading kernel runs and need not wait for
+// pdl_wait.  For the same reason the first kernel of an entry point reads
+// all its inputs so.  What is two launches old or older is safe: a kernel
+// lets the next one start only after its own wait.
 // A kernel in front of one that fills the SMs lets it start (pdl_next) only
 // when its own work is done (kNext false): CTAs that wait keep other streams'
 // kernels out (the 8-frame sweep, started early throughout, was 2% slower).

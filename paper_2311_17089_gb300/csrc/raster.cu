@@ -142,7 +142,7 @@ __device__ __forceinline__ Seg seg_of(const RasterArgs &a, uint32_t c, uint32_t 
     while (hi - lo > 1u) {
         const uint32_t step = (hi - lo + 31u) / 32u, q = lo + (lane + 1u) * step;
         const uint32_t n =
-            __popc(__ballot_sync(0xffffffffu, q < hi && __ldg(a.seg_off + q) <= c));
+            __popc(__ballot_sync(0xffffffffu, q < hi && a.seg_off[q] <= c));
         lo += n * step;
         hi = min(hi, lo + step);
     }
@@ -167,7 +167,7 @@ __device__ __forceinline__ Seg seg_of(const RasterArgs &a, uint32_t c, uint32_t 
 // mean list length D / tiles lies in list_mean_min .. list_mean_max, else
 // the tile kernel.
 __global__ void __launch_bounds__(1024)
-segment_offsets_kernel(const uint32_t *__restrict__ ranges, int tiles, uint32_t resident,
+segment_offsets_kernel(const uint32_t *ranges, int tiles, uint32_t resident,
                        uint32_t *__restrict__ off, uint32_t *__restrict__ seg_len,
                        uint4 *__restrict__ zero, uint32_t n_zero16,
                        uint32_t *__restrict__ use_list, uint32_t list_mean_min,

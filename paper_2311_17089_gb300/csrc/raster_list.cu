@@ -265,14 +265,14 @@ __device__ __forceinline__ void blend_steps(const float4 *__restrict__ cur,
 // p + 256 k + threadIdx.x (a coalesced read); past the mask pass's prefix
 // the thread forms the entry's mask itself.
 __device__ __forceinline__ void load_window(const ListArgs &a, const uint32_t *__restrict__ gl,
-                                            const uint32_t *__restrict__ ml, uint32_t p,
+                                            const uint32_t *ml, uint32_t p,
                                             uint32_t q, int t, uint32_t (&m)[kCullPerThread],
                                             uint32_t (&g)[kCullPerThread]) {
 #pragma unroll
     for (int k = 0; k < kCullPerThread; k++) {
         const uint32_t e = p + (uint32_t)k * 256u + threadIdx.x;
         g[k] = e < q ? __ldg(gl + e) : 0u;
-        m[k] = e >= q ? 0u : e < kMaskPrefix ? __ldg(ml + e) : row_mask_of(a, g[k], t);
+        m[k] = e >= q ? 0u : e < kMaskPrefix ? ml[e] : row_mask_of(a, g[k], t);
     }
 }
 
