@@ -82,13 +82,15 @@ __device__ __forceinline__ float ex2_approx(float x) {
     return y;
 }
 
-// Loads from shared memory at a 32-bit address plus a constant.
+// Loads from shared memory at a 32-bit address plus a constant ("memory":
+// after the stores that wrote it, in the compiler's order too).
 template <int kOff>
 __device__ __forceinline__ float4 lds4(uint32_t p) {
     float4 v;
     asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4 + %5];"
                  : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
-                 : "r"(p), "n"(kOff));
+                 : "r"(p), "n"(kOff)
+                 : "memory");
     return v;
 }
 template <int kOff>
@@ -96,13 +98,17 @@ __device__ __forceinline__ float2 lds2(uint32_t p) {
     float2 v;
     asm volatile("ld.shared.v2.f32 {%0, %1}, [%2 + %3];"
                  : "=f"(v.x), "=f"(v.y)
-                 : "r"(p), "n"(kOff));
+                 : "r"(p), "n"(kOff)
+                 : "memory");
     return v;
 }
 
 __device__ __forceinline__ uint2 lds_offsets(uint32_t p) {
     uint2 v;
-    asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(p));
+    asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];"
+                 : "=r"(v.x), "=r"(v.y)
+                 : "r"(p)
+                 : "memory");
     return v;
 }
 

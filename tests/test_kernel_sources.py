@@ -66,3 +66,16 @@ def test_dependent_kernels_wait_first():
                 assert re.match(r"(using |extern __shared__|__shared__|constexpr |BwdSmem &)", s), (k, s)
             seen += 1
     assert seen >= 12
+
+
+def test_assembly_that_touches_memory_says_so():
+    """Loads, stores, copies and barriers in inline PTX are volatile and name
+    "memory", so that the compiler moves no access across them."""
+    seen = 0
+    for f in os.listdir(CSRC):
+        for m in re.finditer(r"\basm\b(\s+volatile)?\s*\((.*?)\)\s*;", source(f), re.S):
+            text = m.group(2)
+            if re.search(r"\b(ld|st|cp|red|atom|mbarrier|fence|bar|griddepcontrol)\.", text):
+                seen += 1
+                assert m.group(1) and '"memory"' in text, (f, text)
+    assert seen > 20
