@@ -397,7 +397,6 @@ extern "C" int ms_aggregate(const ms_scene_t *scene, const ms_camera_t *cams, in
         a.keys_out = bufs_k[p & 1];
         a.vals_out = bufs_v[p & 1];
         a.n32 = p == 0 ? nullptr : n_small;
-        a.n64 = nullptr;
         a.n_cap = (uint64_t)n;
         a.shift = 8 * p;
         a.hist = hist + 256 * p;

@@ -65,12 +65,8 @@ __device__ __forceinline__ uint32_t block_excl_scan256(uint32_t v, uint32_t *s_w
 __device__ __forceinline__ uint64_t umin64(uint64_t a, uint64_t b) { return a < b ? a : b; }
 
 __device__ __forceinline__ uint64_t pass_count(const PassArgs &a) {
-    uint64_t n = a.n_cap;
-    if (a.n32) n = umin64(n, *a.n32);
-    if (a.n64) n = umin64(n, *a.n64);
-    return n;
+    return a.n32 ? umin64(a.n_cap, *a.n32) : a.n_cap;
 }
-
 
 template <int IPT>
 __global__ void __launch_bounds__(kSortThreads)
@@ -605,8 +601,7 @@ static bool layout(int64_t n, int64_t cap, BinLayout &L) {
     L.dvals_a = take(nn * 4);
     L.dkeys_b = take(nn * 4);
     L.dvals_b = take(nn * 4);
-    L.matrix = take(4 * align256(cap * 4));
-    take((size_t)2 * sort_parts((uint64_t)cap) * 256 * 4);
+    L.matrix = take(4 * align256(cap * 4) + (size_t)2 * sort_parts((uint64_t)cap) * 256 * 4);
     L.zero_begin = o;
     L.tickets = take(16 * 4);
     L.tile_sums = take(kMaxColBlocks * 4);
@@ -657,7 +652,6 @@ int depth_passes(const ms_proj_t *proj, int64_t n, const BinLayout &L, char *w,
         a.keys_out = pass == 3 ? nullptr : dk[pass & 1];
         a.vals_out = pass == 3 ? vals_final : dv[pass & 1];
         a.n32 = pass == 0 ? nullptr : survivors;
-        a.n64 = nullptr;
         a.n_cap = (uint64_t)n;
         a.shift = 8 * pass;
         a.hist = proj->stats + kStatHist + 256 * pass;

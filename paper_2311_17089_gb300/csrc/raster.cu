@@ -46,7 +46,6 @@
 #include <stdint.h>
 
 #include "common.cuh"
-#include "f32x2.cuh"
 #include "tma.cuh"
 #include "raster_ws.cuh"
 #include "raster_list.cuh"
@@ -540,7 +539,7 @@ __device__ __forceinline__ uint32_t ld_volatile(const uint32_t *p) {
 
 // Walk one segment in sub-batches through two staging buffers: while the
 // warps mask, list and blend the records of sub-batch j in one buffer, the
-// bulk copies of sub-batch j + 1 land in the other and the list entries of
+// cp.async copies of sub-batch j + 1 land in the other and the list entries of
 // sub-batch j + 2 are read.  Two CTA barriers per sub-batch: after the block
 // masks, and with the termination test, when every warp is done with
 // sub-batch j.  In local mode (`exact` false) the walk stops as soon as the

@@ -52,7 +52,6 @@ struct PassArgs {
     uint32_t *keys_out;         // nullptr: keys not written
     uint32_t *vals_out;
     const uint32_t *n32;        // device item count (u32) or nullptr
-    const unsigned long long *n64;  // device item count (u64) or nullptr
     uint64_t n_cap;             // count = min(device count, n_cap); or n_cap alone
     int shift;
     const uint32_t *hist;       // [256] digit totals of this pass
@@ -63,7 +62,7 @@ struct PassArgs {
     int ctas_per_sm = 0;               // 0: by the pass's size (below); else this many
 };
 
-// One pass: items [0, count) (count from n32 / n64 / n_cap; only items with
+// One pass: items [0, count) (count from n32 / n_cap; only items with
 // filter[i] > 0 when a filter is given, compacted in index order) are
 // scattered stably by digit (key >> shift) & 255 into keys_out/vals_out.
 // hist holds the digit totals of the items taken; status must hold
