@@ -41,17 +41,18 @@ FP32_LANES_PER_SM = 128    # nominal, for the derived peak shown beside the meas
 OPS_PER_EVAL = 16          # FP32 operations per pixel-Gaussian evaluation
 # FP32 operations per pixel-Gaussian evaluation of the raster backward (an
 # FMA counting as one): the forward's alpha again (power 6, test 2, ex2 and
-# clamp 3), the colour against dL/dC (3), the weight and the recurrences of
-# the colour behind and of T (4), 1 / (1 - alpha) (2), dL/dalpha and
-# dL/dpower (3), and the pixel's share of the record's nine sums (7)
-OPS_PER_BWD_EVAL = 30
+# clamp 3), the weight and the recurrences of the colour so far and of T (6),
+# 1 / (1 - alpha) (2), dC/dalpha over three channels (9), dL/dalpha and
+# dL/dpower (4), and the pixel's share of the record's nine sums (7)
+OPS_PER_BWD_EVAL = 39
 MUFU_LANES_PER_SM = 16     # nominal ex2 results per SM per clock (one ex2 per evaluation)
 PAPER_LEVEL_MIX = (0.95, 0.035, 0.01, 0.005)   # coarse levels under 5% of the Gaussians
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of ncu captures,
 # each with the SHA-256 (first 16 hex digits) of the kernel sources it was
 # taken on: a figure whose sources changed since is reported as stale (null)
-RASTER_DRAM = {"bytes": 33.95e6, "sources": ("raster.cu", "raster_list.cu", "raster_ws.cuh"),
-               "sha16": "d0db282cefbd654c"}   # mean over the 8 frames' raster stages, each frame alone
+RASTER_DRAM = {"bytes": 34.22e6,
+               "sources": ("raster.cu", "raster_list.cu", "raster_ws.cuh", "reach.cuh"),
+               "sha16": "f5d04dd882d30d92"}   # mean over the 8 frames' raster stages, each frame alone
 PROJECT_VIEWS_DRAM = {"bytes": 505.1e6, "sources": ("project.cu", "footprint.cuh"),
                       "sha16": "1e94d3f932b66c6a"}   # the selective sweep's projection launch
 

@@ -81,7 +81,7 @@ typedef enum {
     MS_RASTER_TILE = 1,  /* one thread per pixel; long lists split into
                             segments merged exactly across CTAs             */
     MS_RASTER_LIST = 2,  /* one warp per pixel; only the list entries whose
-                            level-set box reaches the pixel's half row are
+                            reach's box meets the pixel's half row are
                             blended, lanes take consecutive ones, a product
                             scan of (1 - alpha) decides termination        */
     MS_RASTER_GROUP8 = 3,  /* G = 8, 16 or 32 lanes per pixel, 4 consecutive */

@@ -770,9 +770,10 @@ def share_ctas_per_sm(tiles: int, tiles_max: int) -> int:
     beside others (render_views with share_sms), the finest of them having
     tiles_max: 3 for the finest, one fewer for every 4x fewer tiles, at
     least 1, so that the blends leave the SMs room for the other frames'
-    kernels in proportion to their work (on the 1M sweep the 1x, 2x and 4x
-    frames at 3, 2, 1: 1.000-1.008 ms; at 2, 2, 2: 1.040-1.052 ms; at
-    2, 2, 1: 1.009-1.020 ms; every CTA: 1.082-1.088 ms)."""
+    kernels in proportion to their work (the 1M sweep on two scenes, the 1x,
+    2x and 4x frames at 3, 2, 1: 845 and 945 us; at 3, 2, 2: 861 and 965; at
+    2, 2, 2: 896 and 998; at 2, 2, 1: 865 and 1040; at 4, 2, 1: 848 and 945;
+    every CTA: 977 and 1088)."""
     import math
     steps = round(math.log(max(tiles_max, 1) / max(tiles, 1), 4)) if tiles > 0 else 3
     return max(1, 3 - steps)

@@ -897,14 +897,17 @@ extern "C" int ms_raster_ex2(const ms_proj_t *proj, const ms_bins_t *bins,
     // the tile kernel walks quickly, and long ones (all levels, whose
     // pixels end early in lists whose first kMaskPrefix entries the list
     // kernel's mask pass covers whole) to the tile kernel.  Measured on
-    // GB300, 314x208 frames of the 1M-Gaussian scene: selective (3.5k
-    // entries per tile) list 120 against tile 184 us; all levels (19k per
-    // tile) tile 60 us against list 173; the 256x256 single-level frame (70
-    // per tile) is faster on the tile kernel.
-    // The group kernels are chosen only explicitly: the 8-lane one blends a
-    // 314x208 frame alone faster than the tile kernel (176 against 200 us on
-    // GB300) but costs more SM time, and the concurrent 8-frame sweep was
-    // slower with it (1.236 against 1.222 ms).
+    // GB300, this call alone on two 1M-Gaussian scenes: 314x208 selective
+    // (260 tiles, 3.5-4.0k entries each) list 130 and 139 us against tile
+    // 175 and 169; 157x104 (70 tiles) list 66 against tile 117 and 126; all
+    // levels at 314x208 (18k entries) tile 67 and 81 against list 195 and
+    // 221; the 256x256 single-level frame (180 entries) tile 48 against
+    // list 65.  The limits were chosen with an earlier, slower tile kernel:
+    // at 418x277 (486 tiles, 2.5-3.1k entries) the present one would take
+    // 143 and 156 us where the list kernel takes 207 and 198.
+    // The group kernels are chosen only explicitly: on selective frames they
+    // are slower than the kernel chosen here (8 lanes at 314x208: 171 to 191
+    // us).
     const int64_t sms = num_sms();
     const int group = strategy == MS_RASTER_GROUP8    ? 8
                       : strategy == MS_RASTER_GROUP16 ? 16
