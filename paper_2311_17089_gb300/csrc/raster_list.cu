@@ -100,7 +100,7 @@ __device__ __forceinline__ uint32_t window_end(uint32_t p, uint32_t L, uint32_t 
 constexpr uint32_t kMaskPrefix = 16384;
 
 // Bit 2 r + h: the box of the pixels that can accept the entry for Gaussian
-// g (reach_extents; without bounded extents every row), widened by the half
+// g (reach_box; every row where that bounds nothing), widened by the half
 // extents of a half row, reaches the centre of the pixels (16 tx + 8 h +
 // 0..7, 16 ty + r) of tile t = (tx, ty).  The FP32 expression is the one the
 // blend assumes, the same for every half row.
@@ -109,11 +109,11 @@ __device__ __forceinline__ uint32_t row_mask_of(const ListArgs &a, uint32_t g, i
     const float cx0 = (float)(tx * 16) + 4.0f, cx1 = (float)(tx * 16 + 8) + 4.0f;
     MS_DCHECK(g < a.n_rec, a.err);
     if (g >= a.n_rec) g = 0;  // unreachable unless binning reported an error
-    // the centre, the conic and the threshold
-    const float4 u = __ldg(a.rec + 3 * (size_t)g);
-    const float C = __ldg(&a.rec[3 * (size_t)g + 1].x), thr = __ldg(&a.rec[3 * (size_t)g + 2].y);
-    float2 x;
-    if (!reach_extents(u.z, u.w, C, thr, x.x, x.y)) return 0xffffffffu;
+    // the centre and A; the threshold and the half extents (no branch: a
+    // thread's loads for two entries overlap)
+    const float4 u = __ldg(a.rec + 3 * (size_t)g), v = __ldg(a.rec + 3 * (size_t)g + 2);
+    float2 x = make_float2(v.z, v.w);
+    const bool bounded = reach_box(u.z, v.y, x.x, x.y);
     const uint32_t h0 = fabsf(u.x - cx0) <= x.x + kRowHalfX;
     const uint32_t h1 = fabsf(u.x - cx1) <= x.x + kRowHalfX;
     uint32_t m = 0u;
@@ -123,7 +123,7 @@ __device__ __forceinline__ uint32_t row_mask_of(const ListArgs &a, uint32_t g, i
         const uint32_t hit = fabsf(u.y - cy) <= x.y + kRowHalfY;
         m |= (hit & h0) << (2 * r) | (hit & h1) << (2 * r + 1);
     }
-    return m;
+    return bounded ? m : 0xffffffffu;
 }
 
 // The half-row masks of the first kMaskPrefix entries of every tile list,
