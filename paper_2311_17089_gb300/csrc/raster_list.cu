@@ -64,6 +64,7 @@ constexpr int kListSmem = kCntOff + kCullPerThread * kListPixelsPerCta * 4;
 // rounding of the distances (reach.cuh bounds the accepted pixels).
 constexpr float kRowHalfX = 3.5f + 0.0625f;
 constexpr float kRowHalfY = 0.0625f;
+constexpr float kAnywhere = __builtin_huge_valf();
 
 __device__ __forceinline__ float ex2_list(float x) {
     float y;
@@ -99,31 +100,45 @@ __device__ __forceinline__ uint32_t window_end(uint32_t p, uint32_t L, uint32_t 
 // reaches beyond it has its mask formed by the blend's own thread.
 constexpr uint32_t kMaskPrefix = 16384;
 
-// Bit 2 r + h: the box of the pixels that can accept the entry for Gaussian
-// g (reach_box; every row where that bounds nothing), widened by the half
-// extents of a half row, reaches the centre of the pixels (16 tx + 8 h +
-// 0..7, 16 ty + r) of tile t = (tx, ty).  The FP32 expression is the one the
-// blend assumes, the same for every half row.
-__device__ __forceinline__ uint32_t row_mask_of(const ListArgs &a, uint32_t g, int t) {
-    const int tx = t % a.tiles_x, ty = t / a.tiles_x;
-    const float cx0 = (float)(tx * 16) + 4.0f, cx1 = (float)(tx * 16 + 8) + 4.0f;
+// The box of the pixels that can accept Gaussian g (reach_box): centre (x, y)
+// and half extents (z, w), infinite where nothing bounds them.  No branch, so
+// that a thread's loads for two entries overlap.
+__device__ __forceinline__ float4 entry_box(const ListArgs &a, uint32_t g) {
     MS_DCHECK(g < a.n_rec, a.err);
     if (g >= a.n_rec) g = 0;  // unreachable unless binning reported an error
-    // the centre and A; the threshold and the half extents (no branch: a
-    // thread's loads for two entries overlap)
+    // the centre and A; the threshold and the half extents
     const float4 u = __ldg(a.rec + 3 * (size_t)g), v = __ldg(a.rec + 3 * (size_t)g + 2);
     float2 x = make_float2(v.z, v.w);
     const bool bounded = reach_box(u.z, v.y, x.x, x.y);
-    const uint32_t h0 = fabsf(u.x - cx0) <= x.x + kRowHalfX;
-    const uint32_t h1 = fabsf(u.x - cx1) <= x.x + kRowHalfX;
+    return make_float4(u.x, u.y, bounded ? x.x : kAnywhere, bounded ? x.y : kAnywhere);
+}
+
+// Bit 2 r + h: entry_box, widened by the half extents of a half row, reaches
+// the centre of the pixels (16 tx + 8 h + 0..7, 16 ty + r) of tile t =
+// (tx, ty).  The FP32 expressions are the ones the blend assumes, the same
+// for every half row and in row_bit_of.
+__device__ __forceinline__ uint32_t row_mask_of(const ListArgs &a, uint32_t g, int t) {
+    const int tx = t % a.tiles_x, ty = t / a.tiles_x;
+    const float cx0 = (float)(tx * 16) + 4.0f, cx1 = (float)(tx * 16 + 8) + 4.0f;
+    const float4 e = entry_box(a, g);
+    const uint32_t h0 = fabsf(e.x - cx0) <= e.z + kRowHalfX;
+    const uint32_t h1 = fabsf(e.x - cx1) <= e.z + kRowHalfX;
     uint32_t m = 0u;
 #pragma unroll
     for (int r = 0; r < 16; r++) {
         const float cy = (float)(ty * 16 + r) + 0.5f;
-        const uint32_t hit = fabsf(u.y - cy) <= x.y + kRowHalfY;
+        const uint32_t hit = fabsf(e.y - cy) <= e.w + kRowHalfY;
         m |= (hit & h0) << (2 * r) | (hit & h1) << (2 * r + 1);
     }
-    return bounded ? m : 0xffffffffu;
+    return m;
+}
+
+// Bit b of row_mask_of alone, for the CTA of half row b.
+__device__ __forceinline__ uint32_t row_bit_of(const ListArgs &a, uint32_t g, int t, uint32_t b) {
+    const float cx = (float)((t % a.tiles_x) * 16 + (int)(b & 1u) * 8) + 4.0f;
+    const float cy = (float)((t / a.tiles_x) * 16 + (int)(b >> 1)) + 0.5f;
+    const float4 e = entry_box(a, g);
+    return (uint32_t)(fabsf(e.x - cx) <= e.z + kRowHalfX && fabsf(e.y - cy) <= e.w + kRowHalfY) << b;
 }
 
 // The half-row masks of the first kMaskPrefix entries of every tile list,
@@ -263,16 +278,17 @@ __device__ __forceinline__ void blend_steps(const float4 *__restrict__ cur,
 
 // The masks and list indices of window [p, q) for this thread's entries
 // p + 256 k + threadIdx.x (a coalesced read); past the mask pass's prefix
-// the thread forms the entry's mask itself.
+// the thread forms the entry's bit for the CTA's half row itself.
 __device__ __forceinline__ void load_window(const ListArgs &a, const uint32_t *__restrict__ gl,
                                             const uint32_t *ml, uint32_t p,
-                                            uint32_t q, int t, uint32_t (&m)[kCullPerThread],
+                                            uint32_t q, int t, uint32_t b,
+                                            uint32_t (&m)[kCullPerThread],
                                             uint32_t (&g)[kCullPerThread]) {
 #pragma unroll
     for (int k = 0; k < kCullPerThread; k++) {
         const uint32_t e = p + (uint32_t)k * 256u + threadIdx.x;
         g[k] = e < q ? __ldg(gl + e) : 0u;
-        m[k] = e >= q ? 0u : e < kMaskPrefix ? ml[e] : row_mask_of(a, g[k], t);
+        m[k] = e >= q ? 0u : e < kMaskPrefix ? ml[e] : row_bit_of(a, g[k], t, b);
     }
 }
 
@@ -357,10 +373,10 @@ __global__ void __launch_bounds__(256, 4) raster_list_kernel(ListArgs a) {
     // windows [p0, p1) (packed, being blended), [p1, p2) (packed next), [p2, p3)
     uint32_t p0 = 0u, p1 = window_end(0u, L, len), p2 = window_end(p1, L, len);
     uint32_t m[kCullPerThread], g[kCullPerThread];
-    load_window(a, gl, ml, p0, p1, t, m, g);
+    load_window(a, gl, ml, p0, p1, t, (uint32_t)b, m, g);
     uint32_t n_cur = 0u, n_next = 0u;
     pack_window(a, (uint32_t)b, p0, p1, m, g, stage, soff, s_cnt, true, n_cur);
-    load_window(a, gl, ml, p1, p2, t, m, g);
+    load_window(a, gl, ml, p1, p2, t, (uint32_t)b, m, g);
     for (uint32_t wi = 0;; wi++) {
         const uint32_t sb = wi & 1u;
         // this thread's copies of window wi have landed; after the barrier
@@ -373,7 +389,7 @@ __global__ void __launch_bounds__(256, 4) raster_list_kernel(ListArgs a) {
                         s_cnt, px_state.live, n_next) == 0)
             break;  // every pixel has terminated
         const uint32_t p3 = window_end(p2, L, len);
-        load_window(a, gl, ml, p2, p3, t, m, g);
+        load_window(a, gl, ml, p2, p3, t, (uint32_t)b, m, g);
         // blend the window's packed entries two warp steps of 32 at a time
         // (their product scans side by side; 3 or 4 at a time needed more
         // registers than four CTAs per SM leave and were slower)
