@@ -782,8 +782,10 @@ struct Cut {
 
 // Warps per row: kWarps, or what leaves two CTAs per SM their shared memory
 // (16-bit counters: 2 bytes a tile and warp).  Rows: what the SMs hold at
-// once, but enough of them that a row's entries fit 16-bit counts, and no
-// more than the matrix has room for; with room for none (a capacity below
+// once, but enough of them that a row's entries fit 16-bit counts, no more
+// than minimal parts of the capacity fill (CTAs without a row kept the other
+// frames' kernels of an 8-frame sweep waiting), and no more than the matrix
+// has room for; with room for none (a capacity below
 // about a quarter of the tiles) one row of one warp lies in the ranges.
 Cut cut_of(int64_t tiles, int64_t cap, size_t matrix_bytes) {
     Cut c;
@@ -809,7 +811,7 @@ Cut cut_of(int64_t tiles, int64_t cap, size_t matrix_bytes) {
         c.warps = 1;  // little room: a row of one warp needs no offsets
     }
     c.in_ranges = room < 1;
-    c.rows = c.in_ranges ? 1 : std::min(want, room);
+    c.rows = c.in_ranges ? 1 : std::min({want, room, ceil_div(cap, (int64_t)kMinPart * c.warps)});
     // (and, where the count pass sums the columns, a word per tile)
     c.count_smem = std::max<size_t>((size_t)c.warps * c.cnt_words,
                                     tiles <= kFusedTiles ? (size_t)c.stride : 0) * 4;
@@ -879,9 +881,7 @@ int launch_tile_lists(const TileListArgs &t, cudaStream_t st) {
         (rc = ensure_smem_attr(reinterpret_cast<const void *>(rank), kMaxSmem)))
         return rc;
     const unsigned grid = (unsigned)cut.rows, threads = 32u * (unsigned)cut.warps;
-    // no more rows than minimal parts of the capacity
-    pk.fused = t.tiles <= kFusedTiles &&
-               std::min(cut.rows, ceil_div(t.cap, (int64_t)kMinPart * cut.warps)) * t.tiles <= kFusedWords;
+    pk.fused = t.tiles <= kFusedTiles && cut.rows * t.tiles <= kFusedWords;
     pk.ranges = t.ranges;
     if ((rc = cuda_check(launch_after(tile_count_kernel, grid, threads, cut.count_smem, st, pk), "tile counts")))
         return rc;
