@@ -90,16 +90,14 @@ struct PixPair {
     int cntA, cntB;  // entries of the segment each pixel blended through
 };
 
-// Per warp: for kBwdSlots records and the block's 64 pixels (row by row)
-// dL/dpower and the weight w, a pixel's row kBwdSlots + 1 floats long, the
-// second 32 pixels a half bank row further (the warp's halves read them at
-// once); the pixels' dL/dC.
+// Per warp: for kBwdSlots records and the block's 32 pixel pairs (a lane's
+// each) dL/dpower and the weight w as the lanes hold them, a pair's row
+// kBwdSlots + 1 pairs long; the pixels' dL/dC.
 constexpr int kBwdSlots = 16;
-constexpr int kRowF = kBwdSlots + 1;
-constexpr int kHalfF = 32 * kRowF + 16;
+constexpr int kRowP = kBwdSlots + 1;
 struct BwdWarp {
-    float4 d[64];
-    float q[2 * kHalfF - 16], w[2 * kHalfF - 16];
+    f32x2 d[32][4];  // three channels
+    f32x2 q[32 * kRowP], w[32 * kRowP];
     uint16_t list[kBwdBatch];  // records in reach
     uint16_t slot[kBwdSlots];  // the slots' records
 };
@@ -135,54 +133,74 @@ __device__ __forceinline__ bool reaches_block(const float4 r0, float C, float th
 }
 
 // The nine sums of the warp's first n slots, a record per lane pair (lane
-// and lane + 16 take 32 pixels each): the pixels' weights against dL/dC, and
-// the moments of dL/dpower about the record's centre.  Added to the CTA's
-// sums.  (bcx, bcy): the block's centre.  About the record's own centre: the
-// second moments of a splat smaller than a pixel, taken about the block's
-// centre and shifted, are differences of terms a hundred times their size.
+// and lane + 16 take the block's even and odd pixel columns): the pixels'
+// weights against dL/dC, and the moments of dL/dpower about the record's
+// centre.  Added to the CTA's sums.  (bcx, bcy): the block's centre.
+// About the record's own centre: the second moments of a splat smaller than a
+// pixel, taken about the block's centre and shifted, are differences of terms
+// a hundred times their size.  The second moments are summed as a tree (the
+// pairs' two rows, rows 2 and 1 apart, columns 4, 2 and 1 apart): the chain
+// to scales and rotations amplifies their last bits, a thousandfold for the
+// worst of 1M Gaussians.
 __device__ __forceinline__ void add_slots(const BwdWarp &wp, uint32_t n, const float4 *rec,
                                           float bcx, float bcy, float (*acc)[kG2 + 1]) {
     const uint32_t lane = threadIdx.x & 31u, r = lane & 15u, h = lane >> 4;
-    const float *q = wp.q + h * kHalfF + r, *w = wp.w + h * kHalfF + r;
-    const float4 *d = wp.d + 32 * h;
+    const f32x2 *q = wp.q + h * kRowP + r, *w = wp.w + h * kRowP + r;
     // lanes without a record sum slots that nothing reads; their centre is
     // any staged record's
     const uint32_t j = r < n ? wp.slot[r] : wp.slot[0];
     const float4 r0 = rec[3 * j];
     const float2 r1 = *reinterpret_cast<const float2 *>(rec + 3 * j + 1);
-    float X[8], XX[8];  // pixel columns from the record's centre
+    f32x2 dy[4];
 #pragma unroll
-    for (int x = 0; x < 8; x++) {
-        X[x] = (bcx + ((float)x - 3.5f)) - r0.x;
-        XX[x] = X[x] * X[x];
-    }
-    float m0 = 0.0f, mx = 0.0f, my = 0.0f, mxx = 0.0f, mxy = 0.0f, myy = 0.0f;
-    float w0 = 0.0f, w1 = 0.0f, w2 = 0.0f;
-    const float y0 = bcy + (h ? 0.5f : -3.5f);
+    for (int y = 0; y < 4; y++)
+        dy[y] = sub2(pack2(bcy + ((float)y - 3.5f), bcy + ((float)y + 0.5f)), splat2(r0.y));
+    float m0 = 0.0f, mx = 0.0f, my = 0.0f;
+    f32x2 w0 = 0ull, w1 = 0ull, w2 = 0ull;
+    float mxx[4], mxy[4], myy[4];  // per column
 #pragma unroll
-    for (int row = 0; row < 4; row++) {
-        float s0 = 0.0f, s1 = 0.0f, s2 = 0.0f;
+    for (int i = 0; i < 4; i++) {
+        const float dx = (bcx + ((float)(2 * i) - 3.5f + (float)h)) - r0.x;
+        const float cx = -0.5f * dx * dx;
+        float s[4], sy[4], syy[4];
 #pragma unroll
-        for (int x = 0; x < 8; x++) {
-            const int p = row * 8 + x;
-            const float qv = q[p * kRowF], wv = w[p * kRowF];
-            const float4 dv = d[p];
-            s0 += qv;
-            s1 = fmaf(qv, X[x], s1);
-            s2 = fmaf(qv, XX[x], s2);
-            w0 = fmaf(wv, dv.x, w0);
-            w1 = fmaf(wv, dv.y, w1);
-            w2 = fmaf(wv, dv.z, w2);
+        for (int y = 0; y < 4; y++) {
+            const int p = y * 8 + 2 * i;  // pair of column 2 i + h
+            const f32x2 qv = q[p * kRowP], wv = w[p * kRowP];
+            const ulonglong2 d01 = *reinterpret_cast<const ulonglong2 *>(wp.d[p + h]);
+            w0 = fma2(wv, d01.x, w0);
+            w1 = fma2(wv, d01.y, w1);
+            w2 = fma2(wv, wp.d[p + h][2], w2);
+            const f32x2 qy = mul2(qv, dy[y]);
+            float lo, hi;
+            unpack2(qv, lo, hi);
+            s[y] = lo + hi;
+            unpack2(qy, lo, hi);
+            sy[y] = lo + hi;
+            unpack2(mul2(qy, dy[y]), lo, hi);
+            syy[y] = lo + hi;
         }
-        const float Y = (y0 + (float)row) - r0.y;
-        m0 += s0;
-        mx += s1;
-        mxx += s2;
-        my = fmaf(Y, s0, my);
-        mxy = fmaf(Y, s1, mxy);
-        myy = fmaf(Y * Y, s0, myy);
+        const float sx = (s[0] + s[2]) + (s[1] + s[3]);
+        m0 += sx;
+        mx = fmaf(sx, dx, mx);
+        my += (sy[0] + sy[2]) + (sy[1] + sy[3]);
+        mxx[i] = (__fmul_rn(s[0], cx) + __fmul_rn(s[2], cx)) + (__fmul_rn(s[1], cx) + __fmul_rn(s[3], cx));
+        mxy[i] = (__fmul_rn(sy[0], dx) + __fmul_rn(sy[2], dx)) + (__fmul_rn(sy[1], dx) + __fmul_rn(sy[3], dx));
+        myy[i] = (syy[0] + syy[2]) + (syy[1] + syy[3]);
     }
-    float v[kG2] = {m0, mx, my, mxx, mxy, myy, w0, w1, w2};
+    float wl[3], wh[3];
+    unpack2(w0, wl[0], wh[0]);
+    unpack2(w1, wl[1], wh[1]);
+    unpack2(w2, wl[2], wh[2]);
+    float v[kG2] = {m0,
+                    mx,
+                    my,
+                    (mxx[0] + mxx[2]) + (mxx[1] + mxx[3]),
+                    (mxy[0] + mxy[2]) + (mxy[1] + mxy[3]),
+                    (myy[0] + myy[2]) + (myy[1] + myy[3]),
+                    wl[0] + wh[0],
+                    wl[1] + wh[1],
+                    wl[2] + wh[2]};
 #pragma unroll
     for (int k = 0; k < kG2; k++) v[k] += __shfl_xor_sync(0xffffffffu, v[k], 16);
     if (r >= n) return;
@@ -192,7 +210,7 @@ __device__ __forceinline__ void add_slots(const BwdWarp &wp, uint32_t n, const f
     if (h == 0) {
         atomicAdd(&acc[j][0], ca * v[1] + cb * v[2]);
         atomicAdd(&acc[j][1], cb * v[1] + cc * v[2]);
-        atomicAdd(&acc[j][2], -0.5f * v[3]);
+        atomicAdd(&acc[j][2], v[3]);
         atomicAdd(&acc[j][3], -v[4]);
         atomicAdd(&acc[j][4], -0.5f * v[5]);
         acc[j][kG2] = 1.0f;
@@ -212,7 +230,7 @@ __device__ __forceinline__ void add_slots(const BwdWarp &wp, uint32_t n, const f
 // record per lane, instead of nine reductions across the warp per record
 // (12 shuffles and about 70 instructions).  With records culled by their
 // level set instead of its box, and cp.async staging: the 4-view batch of 1M
-// Gaussians (1256x832, 314x208, 78x52, 19x13) 820 -> 650 us; 590 with the
+// Gaussians (1256x832, 314x208, 78x52, 19x13) 820 -> 635 us; 590 with the
 // colour behind kept as one product and the moments about the block's
 // centre, which lost precision (add_slots and the head of this file).
 __global__ void __launch_bounds__(kBwdThreads, 4)
@@ -231,7 +249,7 @@ raster_bwd_kernel(const __grid_constant__ BwdArgs args) {
     const int lyA = (wid >> 1) * 8 + (lane >> 3), lyB = lyA + 4;
     const int fA = fwd_index(lx, lyA), fB = fwd_index(lx, lyB);
     for (int i = tid; i < kBwdBatch * (kG2 + 1); i += kBwdThreads) (&sm.acc[0][0])[i] = 0.0f;
-    for (int i = lane; i < (int)(sizeof(wp.q) / 4); i += 32) wp.q[i] = wp.w[i] = 0.0f;
+    for (int i = lane; i < 32 * kRowP; i += 32) wp.q[i] = wp.w[i] = 0ull;
     if (tid == 0) {
         uint32_t run = 0;
         for (int k = 0; k < args.n_views; k++) {
@@ -304,7 +322,6 @@ raster_bwd_kernel(const __grid_constant__ BwdArgs args) {
                     st[h][9] = a.dl[2 * plane + p];
                 }
             }
-            wp.d[lane + 32 * h] = make_float4(st[h][7], st[h][8], st[h][9], 0.0f);
         }
         pp.T = pack2(st[0][0], st[1][0]);
         pp.F0 = pack2(st[0][1], st[1][1]);
@@ -316,6 +333,9 @@ raster_bwd_kernel(const __grid_constant__ BwdArgs args) {
         pp.d0 = pack2(st[0][7], st[1][7]);
         pp.d1 = pack2(st[0][8], st[1][8]);
         pp.d2 = pack2(st[0][9], st[1][9]);
+        wp.d[lane][0] = pp.d0;
+        wp.d[lane][1] = pp.d1;
+        wp.d[lane][2] = pp.d2;
         pp.cntA = (int)cnt[0];
         pp.cntB = (int)cnt[1];
         const float fx = (float)px + 0.5f;
@@ -399,14 +419,9 @@ raster_bwd_kernel(const __grid_constant__ BwdArgs args) {
                 const f32x2 t2 = fma2(sub2(pp.C2, pp.F2), nio, mul2(pp.T, c2));
                 const f32x2 dal = fma2(pp.d2, t2, fma2(pp.d1, t1, mul2(pp.d0, t0)));
                 pp.T = mul2(pp.T, om);
-                float q0, q1, w0, w1;
-                unpack2(mul2(dal, ag), q0, q1);  // dL/dpower
-                unpack2(w, w0, w1);
-                const uint32_t at = (uint32_t)lane * kRowF + ns;
-                wp.q[at] = q0;
-                wp.q[kHalfF + at] = q1;
-                wp.w[at] = w0;
-                wp.w[kHalfF + at] = w1;
+                const uint32_t at = (uint32_t)lane * kRowP + ns;
+                wp.q[at] = mul2(dal, ag);  // dL/dpower
+                wp.w[at] = w;
                 if (lane == 0) wp.slot[ns] = (uint16_t)j;
                 if (++ns == kBwdSlots) {
                     __syncwarp();
