@@ -222,13 +222,13 @@ __device__ __forceinline__ void add_slots(const BwdWarp &wp, uint32_t n, const f
     }
 }
 
-// Bound by instruction issue with the warps that 54 KB and 128 registers a
-// CTA's thread leave: 416M warp instructions at 55% of the slots, 15 of 64
-// warps resident (the 4-view batch below).  A record costs a warp about 65
-// instructions for its 64 pixels' gradients and 24 for the nine sums over
-// them: those are 9 x 64 products with per-pixel factors, formed 16 records at a time with a
-// record per lane, instead of nine reductions across the warp per record
-// (12 shuffles and about 70 instructions).  With records culled by their
+// Bound by instruction issue with the warps that 54 KB a CTA and 126
+// registers a thread leave: 385M warp instructions at 52% of the slots, 15 of
+// 64 warps resident (the 4-view batch below).  A record costs a warp about 65
+// instructions for its 64 pixels' gradients and 20 for the nine sums over
+// them: those are 9 x 64 products with per-pixel factors, formed 16 records
+// at a time with a record per lane, instead of nine reductions across the
+// warp per record (12 shuffles and about 70 instructions).  With records culled by their
 // level set instead of its box, and cp.async staging: the 4-view batch of 1M
 // Gaussians (1256x832, 314x208, 78x52, 19x13) 820 -> 635 us; 590 with the
 // colour behind kept as one product and the moments about the block's
