@@ -398,7 +398,8 @@ int ms_bin_noalloc(const ms_proj_t *proj, int64_t n, const ms_camera_t *cam,
  * Copy the counts of a finished ms_bin to the host (synchronises
  * `stream`).  Returns MS_ERR_BOUNDS if an index check of the debug build
  * failed (in ms_bin or in an ms_raster that used these bins),
- * MS_ERR_TIMEOUT if a bounded wait gave up, MS_ERR_CAPACITY if D exceeded
+ * MS_ERR_TIMEOUT if a bounded wait gave up or the projection held tiles that
+ * the binned frame does not have (another camera's; the lists are not valid), MS_ERR_CAPACITY if D exceeded
  * the capacity (*d_needed tells how many are needed), else MS_OK.  Either
  * pointer may be NULL.
  */
